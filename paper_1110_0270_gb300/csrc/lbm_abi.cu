@@ -97,6 +97,10 @@ void fill_params(const lbm_config* cfg, int nsm, Params& p) {
     // 2^-49 rho: below that the state is at equilibrium as far as the
     // storage can tell, and the LBGK step is taken as for Delta S < 1e-15
     p.elbm_skip_rel = cfg->precision == LBM_FP64 ? 0.0 : 0x1p-48;
+    p.elbm_thr[0] = 1e-15f;
+    p.elbm_thr[1] = (float)p.elbm_skip_rel;
+    p.beta2[0] = (float)(2.0 * p.beta);
+    p.beta2[1] = (float)(2.0 * p.beta - (double)p.beta2[0]);
     p.lim_alpha = cfg->lim_alpha;
     p.lim_k = cfg->lim_k;
     p.lim_dst = cfg->lim_dst;
@@ -146,7 +150,7 @@ struct Layout {
     int Q, pitch;
     int64_t plane;
     size_t f_off, f_bytes, cnt_off, cand_f_off, cand_ds_off, cand_site_off, cand_sel_off,
-        field_off, red_off, staging_off, total;
+        field_off, red_off, slot_off, staging_off, total;
     int cand_cap;
 };
 
@@ -176,6 +180,8 @@ Layout layout(const lbm_config* c) {
     off += c->collision == LBM_MEDIAN ? align_up(N * math_bytes(c->precision)) : 0;
     L.red_off = off;  // kRedSlots sums + kRedSlots counts + E
     off += reduces(c->collision) ? align_up((2 * kRedSlots + 8) * sizeof(double)) : 0;
+    L.slot_off = off;
+    off += c->collision == LBM_ELBM ? kStatSlots * kStatStride * sizeof(unsigned long long) : 0;
     L.staging_off = off;
     off += align_up(3 * N * 8);
     L.total = off;
@@ -273,6 +279,8 @@ __global__ void __launch_bounds__(256) enstrophy_kernel(int nx, int ny, int px, 
 
 lbm_status reset_counters(lbm_ctx* ctx, cudaStream_t s) {
     LBM_CK(ctx, cudaMemsetAsync(ctx->p.counters, 0, CNT_WORDS * 4 + ST_WORDS * 8, s));
+    if (ctx->p.stat_slots)
+        LBM_CK(ctx, cudaMemsetAsync(ctx->p.stat_slots, 0, kStatSlots * kStatStride * sizeof(unsigned long long), s));
     return LBM_OK;
 }
 
@@ -483,10 +491,13 @@ lbm_status lbm_create(const lbm_config* cfg, void* dev_mem, size_t bytes, lbm_ct
         p.lim_E = p.red + 2 * kRedSlots;
         p.lim_E_f = (float*)(p.lim_E + 1);
     }
+    if (cfg->collision == LBM_ELBM) p.stat_slots = (unsigned long long*)(ctx->base + L.slot_off);
     ctx->staging = (double*)(ctx->base + L.staging_off);
     cudaError_t e = cudaMemset(ctx->base + L.cnt_off, 0, align_up(CNT_WORDS * 4 + ST_WORDS * 8 + 64));
     if (e == cudaSuccess && reduces(cfg->collision))
         e = cudaMemset(ctx->base + L.red_off, 0, (2 * kRedSlots + 8) * sizeof(double));
+    if (e == cudaSuccess && p.stat_slots)
+        e = cudaMemset(p.stat_slots, 0, kStatSlots * kStatStride * sizeof(unsigned long long));
     const char* where = "cudaMemset of the counters";
     if (e == cudaSuccess) {
         e = build_step_graph(ctx);
@@ -660,7 +671,15 @@ lbm_status lbm_stats_get(lbm_ctx* ctx, lbm_stats* out, void* stream) {
     unsigned long long st[ST_WORDS];
     LBM_CK(ctx, cudaMemcpyAsync(cnt, ctx->p.counters, sizeof cnt, cudaMemcpyDeviceToHost, S(stream)));
     LBM_CK(ctx, cudaMemcpyAsync(st, ctx->p.stats, sizeof st, cudaMemcpyDeviceToHost, S(stream)));
+    unsigned long long slots[kStatSlots * kStatStride] = {0};
+    if (ctx->p.stat_slots)
+        LBM_CK(ctx, cudaMemcpyAsync(slots, ctx->p.stat_slots, sizeof slots, cudaMemcpyDeviceToHost, S(stream)));
     LBM_CK(ctx, cudaStreamSynchronize(S(stream)));
+    for (int k = 0; k < kStatSlots; ++k) {
+        const unsigned long long* v = slots + k * kStatStride;
+        for (int w : {ST_ELBM_SOLVED, ST_ELBM_SKIPPED, ST_ELBM_FALLBACK, ST_ELBM_ITERS}) st[w] += v[w];
+        if (v[ST_ELBM_ITERS_MAX] > st[ST_ELBM_ITERS_MAX]) st[ST_ELBM_ITERS_MAX] = v[ST_ELBM_ITERS_MAX];
+    }
     std::memset(out, 0, sizeof *out);
     out->steps = ctx->t;
     out->candidates_last = (ctx->t > 0 && limiter(ctx->cfg.collision)) ? cnt[CNT_NVALID] : 0;

@@ -101,7 +101,13 @@ __device__ __forceinline__ void batch_tile(const Params& sp, const BatchItem& it
     for (int r = 0; r < rows; ++r) {
         const int x = Q == 9 ? it.x0 + (tid & ((1 << log2x) - 1)) : it.x0 + r * kBatchThreads + tid;
         const int y = Q == 9 ? it.y0 + r * th + (tid >> log2x) : 0;
-        if (x < sp.nx && y < sp.ny) {
+        if constexpr (kElbmWarp<ST, COLL>) {
+            const bool valid = x < sp.nx && y < sp.ny;
+            if (odd)
+                elbm_update<Q, ST, true>(sp, x, y, valid, e_code, e_iters);
+            else
+                elbm_update<Q, ST, false>(sp, x, y, valid, e_code, e_iters);
+        } else if (x < sp.nx && y < sp.ny) {
             if (odd)
                 site_update<Q, ST, COLL, true>(sp, x, y, e_code, e_iters, acc);
             else
@@ -196,10 +202,11 @@ __device__ __forceinline__ void batch_dispatch(const Params& sp, const BatchItem
 
 // Resident CTAs per SM each kernel is compiled for (0: no register cap), in
 // the 16/32-bit formats: the streaming set six (40 registers), the limiters
-// five (48; at 40 they spilled over 1 KB, mostly on the fix-up paths); ELBM
-// and FP64 storage uncapped.
+// five (48; at 40 they spilled over 1 KB, mostly on the fix-up paths), ELBM
+// three (80; a batch of 32 instances 5.50 ms for 20 steps against 5.62 at
+// four and 5.69 at five); FP64 storage uncapped.
 template <class ST, int SET>
-constexpr int kBatchMinBlocks = sizeof(typename ST::T) == 8 ? 0 : (SET == kSetStream ? 6 : (SET == kSetLimiter ? 5 : 0));
+constexpr int kBatchMinBlocks = sizeof(typename ST::T) == 8 ? 0 : (SET == kSetStream ? 6 : (SET == kSetLimiter ? 5 : 3));
 
 // Completion of a run of `count` items of one instance and step (all
 // threads): their stores are made visible, the instance's item counter

@@ -20,7 +20,7 @@
 //                   post-collision one (FP32 / FP64 storage).
 #pragma once
 
-#include "lbm_device.cuh"
+#include "lbm_elbm_f32.cuh"
 
 namespace lbm {
 
@@ -144,16 +144,8 @@ __device__ __forceinline__ void collide_site(const Params& p, int x, int y, cons
         e_code = out.code;
         e_iters = out.iters;
         const double ab = out.alpha * p.beta;
-        if constexpr (sizeof(T) == 8) {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) F[i] = fd[i] + ab * Dd[i];
-        } else {
-            // F = f + alpha beta (f* - f) rounds to FP32 (or 16 bits) anyway:
-            // the product in FP32 on the FP64 difference, no FP64 update
-            const float abf = (float)ab;
-#pragma unroll
-            for (int i = 0; i < Q; ++i) F[i] = fmaf(abf, (float)Dd[i], f[i]);
-        }
+        for (int i = 0; i < Q; ++i) F[i] = T(fd[i] + ab * Dd[i]);
     } else if ((COLL >= LBM_SMOOTH && COLL <= LBM_THRESHOLD) || COLL == LBM_ENSEMBLE_LAGGED) {
         // Sections 4.2-4.4: f -> f* + phi(Delta S) (f - f*), then LBGK, i.e.
         // F = f* + (1 - 2 beta) phi (f - f*); the threshold limiter's phi is
@@ -723,6 +715,32 @@ __device__ __forceinline__ void site_update(const Params& p, int x, int y, int& 
         store_general<Q, ST, ODD, DEV>(p, x, y, F);
 }
 
+// ELBM in FP32 arithmetic runs on whole warps (elbm_warp).
+template <class ST, int COLL>
+constexpr bool kElbmWarp = COLL == LBM_ELBM && sizeof(typename ST::T) == 4;
+
+// Its step of a warp's sites (every lane calls it; valid: the lane has a site).
+template <int Q, class ST, bool ODD>
+__device__ __forceinline__ void elbm_update(const Params& p, int x, int y, bool valid, int& e_code, int& e_iters) {
+    float f[Q], F[Q];
+    const bool interior = x > 0 && x < p.nx - 1 && (Q == 3 || (y > 0 && y < p.ny - 1));
+    const int o = y * p.pitch + x;
+    if (Q == 9 && p.diffusive && !interior) valid = false;  // diffusive_wall_kernel's sites
+    if (valid) {
+        if (interior)
+            load_interior<Q, ST, ODD>(p, o, f);
+        else
+            load_general<Q, ST, ODD>(p, x, y, f);
+    }
+    elbm_warp<Q>(p, valid, f, F, e_code, e_iters);
+    if (valid) {
+        if (interior)
+            store_interior<Q, ST, ODD>(p, o, F);
+        else
+            store_general<Q, ST, ODD>(p, x, y, F);
+    }
+}
+
 // Warp-aggregated ELBM counters (all 32 lanes of the warp call this).
 __device__ __forceinline__ void elbm_stats(const Params& p, int e_code, int e_iters) {
     unsigned solved = __reduce_add_sync(0xffffffffu, e_code == 0 ? 1u : 0u);
@@ -731,11 +749,15 @@ __device__ __forceinline__ void elbm_stats(const Params& p, int e_code, int e_it
     unsigned iters = __reduce_add_sync(0xffffffffu, (unsigned)e_iters);
     unsigned itmax = __reduce_max_sync(0xffffffffu, (unsigned)e_iters);
     if (lane_id() == 0) {
-        if (solved) atomicAdd(&p.stats[ST_ELBM_SOLVED], (unsigned long long)solved);
-        if (skipped) atomicAdd(&p.stats[ST_ELBM_SKIPPED], (unsigned long long)skipped);
-        if (fallback) atomicAdd(&p.stats[ST_ELBM_FALLBACK], (unsigned long long)fallback);
-        if (iters) atomicAdd(&p.stats[ST_ELBM_ITERS], (unsigned long long)iters);
-        if (itmax) atomicMax(&p.stats[ST_ELBM_ITERS_MAX], (unsigned long long)itmax);
+        unsigned long long* st =
+            p.stat_slots ? p.stat_slots + ((blockIdx.y * gridDim.x + blockIdx.x) % kStatSlots) * kStatStride : p.stats;
+        if (solved) atomicAdd(&st[ST_ELBM_SOLVED], (unsigned long long)solved);
+        if (skipped) atomicAdd(&st[ST_ELBM_SKIPPED], (unsigned long long)skipped);
+        if (fallback) atomicAdd(&st[ST_ELBM_FALLBACK], (unsigned long long)fallback);
+        if (iters) atomicAdd(&st[ST_ELBM_ITERS], (unsigned long long)iters);
+        // (the largest count only grows: most warps find theirs no larger)
+        if (itmax && itmax > *(volatile unsigned long long*)&st[ST_ELBM_ITERS_MAX])
+            atomicMax(&st[ST_ELBM_ITERS_MAX], (unsigned long long)itmax);
     }
 }
 
@@ -780,15 +802,17 @@ __device__ __forceinline__ void block_sum_to_slots(const Params& p, T a, T b, bo
 // Ehrenfest and positivity: eight (32 registers, a few bytes of spills;
 // measured 4% faster than six); median: six (at 32 registers its FP32
 // Delta S spills ~200 bytes) and the Section 4.2-4.4 limiters (four bytes
-// of spills).  0 leaves the choice to the compiler (LBGK and
-// MRT fit in 32-38 registers by themselves; ELBM and FP64 storage are not
-// capped).
+// of spills).  ELBM: five (48 registers; the 2049^2 step 121 us against 126
+// at four and 144 at three; its spills are around the out-of-line solves).
+// 0 leaves the choice to the compiler (LBGK and
+// MRT fit in 32-38 registers by themselves; FP64 storage is not capped).
 template <class ST, int COLL>
 constexpr int kMinBlocks =
     (COLL == LBM_ELBM && sizeof(typename ST::T) == 8)
         ? 2  // 128 registers: two CTAs per SM also near rest, where the step streams
         : sizeof(typename ST::T) != 4
         ? 0
+        : COLL == LBM_ELBM ? 5
         : (COLL == LBM_EHRENFEST || COLL == LBM_POSITIVITY || COLL == LBM_MRT_LIMITER)
               ? 8
               : (COLL == LBM_MEDIAN || (COLL >= LBM_SMOOTH && COLL <= LBM_THRESHOLD) || COLL == LBM_ENSEMBLE_LAGGED)
@@ -848,7 +872,10 @@ __global__ void __launch_bounds__(kBlockX* kBlockY, kMinBlocks<ST, COLL>) step_k
     if (kSitePrefetch<Q, ST, COLL>) prefetch_ahead<Q, ST>(p, kBlockX, 8);
     int e_code = -1, e_iters = 0;
     typename ST::T acc = 0;
-    if (x < p.nx && y < p.ny) site_update<Q, ST, COLL, ODD>(p, x, y, e_code, e_iters, acc);
+    if constexpr (kElbmWarp<ST, COLL>)
+        elbm_update<Q, ST, ODD>(p, x, y, x < p.nx && y < p.ny, e_code, e_iters);
+    else if (x < p.nx && y < p.ny)
+        site_update<Q, ST, COLL, ODD>(p, x, y, e_code, e_iters, acc);
     if (COLL == LBM_ELBM) elbm_stats(p, e_code, e_iters);
     if (COLL == LBM_THRESHOLD) block_sum_to_slots<typename ST::T>(p, acc, 0, false);
     if (COLL == LBM_ENSEMBLE_LAGGED)

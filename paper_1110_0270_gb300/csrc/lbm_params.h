@@ -29,6 +29,11 @@ enum Counter {
     CNT_WORDS = 8
 };
 constexpr int kRedSlots = 1024;  // partial-sum slots (spread the atomics)
+// ELBM counters: 64 copies of the statistics, one 128-byte line each, picked
+// by CTA.  One copy took three atomics of every warp on three addresses, and
+// that L2 slice (81% busy, the others 12%), not the arithmetic, set the time
+// of the 2049^2 FP32 step (275 us).
+constexpr int kStatSlots = 64, kStatStride = 16;
 
 enum Stat {
     ST_LIMITED = 0,
@@ -57,6 +62,8 @@ struct Params {
     double elbm_eps;
     int elbm_max_iter, elbm_norm, elbm_fallback;
     double elbm_skip_rel;  // near-equilibrium skip: Delta S < 1e-15 + elbm_skip_rel * rho
+    float elbm_thr[2];     // FP32 copies of that threshold's two terms
+    float beta2[2];        // 2 beta as the sum of two floats
     // Sections 4.2-4.4 limiters
     double lim_alpha, lim_k, lim_dst, lim_delta0;
     double* red;      // kRedSlots partial sums (+ kRedSlots counts), zero between steps
@@ -71,6 +78,7 @@ struct Params {
     // scratch
     unsigned* counters;              // CNT_WORDS words
     unsigned long long* stats;       // ST_WORDS words
+    unsigned long long* stat_slots;  // ELBM: kStatSlots x kStatStride words added to stats (NULL: none)
     int cand_cap;                    // capacity of the candidate list
     void* cand_f;                    // [Q][cand_cap] arithmetic type
     double* cand_ds;                 // [cand_cap] FP64 Delta S (-1: not a candidate)
