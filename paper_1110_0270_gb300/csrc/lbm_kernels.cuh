@@ -882,6 +882,39 @@ __global__ void __launch_bounds__(kBlockX* kBlockY, kMinBlocks<ST, COLL>) step_k
         block_sum_to_slots<typename ST::T>(p, acc, e_code == 1 ? typename ST::T(1) : typename ST::T(0), true);
 }
 
+// ELBM on a D1Q3 line in FP64 storage, four lanes per site (elbm_lanes): lane
+// q < 3 of a group owns population q, its address included.  CTAs of one
+// warp (eight sites), so that a line of a few hundred sites spreads over the
+// SMs.
+constexpr int kLaneSites = 8;  // sites per warp
+
+template <class ST, bool ODD>
+__global__ void __launch_bounds__(32) elbm_lanes_step(Params p) {
+    pdl_enter();
+    using L = Lat<3>;
+    constexpr int G = ElbmLanes<3>::G;
+    const int lane = threadIdx.x, q = lane & (G - 1);
+    const int x = blockIdx.x * kLaneSites + lane / G;
+    const bool valid = x < p.nx, act = valid && q < 3;
+    double f = 0.0, lidc;
+    int64_t r = 0;
+    if (act) {
+        r = aa_address<3, double>(p, x, 0, q, ODD, lidc);
+        f = ((const double*)p.f)[r];
+    }
+    const ElbmLane e = elbm_lanes<3>(p, f, valid);
+    if (valid && q == 0 && (!(e.rho > 0.0) || !(fabs(e.ux) < 1e30)))
+        if (*(volatile unsigned*)&p.counters[CNT_DIVERGED] == 0u) atomicExch(&p.counters[CNT_DIVERGED], 1u);
+    double F = f + (e.alpha * p.beta) * e.D;
+    // the rest population as rho minus the others, then F_opp to this lane's address
+    const double other = q == L::rest || q >= 3 ? 0.0 : F;
+    const double sum = group_sum<G>(other);
+    if (q == L::rest) F = e.rho - sum;
+    F = __shfl_sync(0xffffffffu, F, (lane & ~(G - 1)) + (q < 3 ? L::opp(q) : q));
+    if (act) ((double*)p.f)[r] = F;
+    elbm_stats(p, valid && q == 0 ? e.code : -1, valid && q == 0 ? e.iters : 0);
+}
+
 // Two sites per thread (x0 = 2t, x0 + 1): every population plane moves with
 // one aligned 32-bit access per thread holding the pair (and one packed
 // conversion).  In odd steps the planes with v_x = +-1 are one element off;
@@ -2310,6 +2343,11 @@ inline dim3 site_grid(const Params& p, dim3 block) {
 
 inline dim3 site_block(int Q) { return Q == 3 ? dim3(256, 1) : dim3(kBlockX, kBlockY); }
 
+// A line up to this long takes four lanes per site in FP64 ELBM: the groups of
+// lanes run a shorter chain on four times the warps (800 sites: 20.6 us a step
+// against 49; 20000 sites, where the warps fill the FP64 pipes: 58 us against 55).
+constexpr int kElbmLaneMost = 16000;
+
 template <int Q, class ST, int COLL>
 cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
     // two sites per thread where every row starts on a pair boundary (the
@@ -2323,6 +2361,10 @@ cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
                             s, p);
         }
     }
+    if constexpr (Q == 3 && COLL == LBM_ELBM && sizeof(typename ST::T) == 8)
+        if (p.nx <= kElbmLaneMost)
+            return launch_p(odd ? elbm_lanes_step<ST, true> : elbm_lanes_step<ST, false>,
+                            dim3((p.nx + kLaneSites - 1) / kLaneSites), dim3(32), s, p);
     dim3 b = site_block(Q);
     if (Q == 3) {
         // a D1Q3 line has few sites (the 800-site tube): spread them over the

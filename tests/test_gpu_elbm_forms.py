@@ -61,3 +61,13 @@ def test_fp32_few_hard_sites_per_warp():
     f0 = f0 * WL.lognormal_factors(f0.shape, 6, 1e-3)
     f0[2, 4, 3] = f0[7, 4, 17] = f0[1, 6, 40] = 1e-9
     assert one_step(cfg, f0.astype(np.float32).astype(np.float64)) < TOL32
+
+
+@pytest.mark.parametrize("nx", [1, 2, 7, 8, 9, 33, 800, 15999, 16001])
+@pytest.mark.parametrize("width", [1e-3, 0.3])
+def test_fp64_line(nx, width):
+    """FP64 (1e-12: the reordered sums and the solve's own 1e-15)."""
+    cfg = dict(lattice="D1Q3", nx=nx, ny=1, bc="ends", collision="elbm", precision="fp64", beta=0.95)
+    fl = WL.random_fields(1, nx, 3, 0.05, 0.1)
+    f0 = O.init_equilibrium(cfg, fl["rho"], fl["ux"], None)
+    assert one_step(cfg, f0 * WL.lognormal_factors(f0.shape, 4, width)) < 1e-12
