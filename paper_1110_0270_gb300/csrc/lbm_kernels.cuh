@@ -1176,23 +1176,57 @@ __device__ __forceinline__ int pick_digit(const unsigned* hist, unsigned& rem, b
     return digit;
 }
 
-// Sum over the CTA, returned to every thread (every thread calls it).
-__device__ __forceinline__ double block_sum(double v) {
-    __shared__ double part[32];
-    __shared__ double total;
+// Sums over the CTA of a and b, returned to every thread (every thread calls it).
+__device__ __forceinline__ void block_sum2(double& a, double& b) {
+    __shared__ double part[2][32];
     const int t = threadIdx.y * blockDim.x + threadIdx.x;
     const int nw = (blockDim.x * blockDim.y + 31) >> 5;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();  // part / total free from a previous call
-    if ((t & 31) == 0) part[t >> 5] = v;
-    __syncthreads();
-    if (t < 32) {
-        double u = t < nw ? part[t] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
-        if (t == 0) total = u;
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    __syncthreads();  // part free from a previous call
+    if ((t & 31) == 0) {
+        part[0][t >> 5] = a;
+        part[1][t >> 5] = b;
     }
     __syncthreads();
-    return total;
+    // every warp adds the warps' sums (at most 32) by itself
+    const int l = t & 31;
+    a = l < nw ? part[0][l] : 0.0;
+    b = l < nw ? part[1][l] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+}
+
+// Inclusive prefix sums of c and v over the 256 threads of the CTA in thread
+// order (every thread calls it).
+__device__ __forceinline__ void block_scan2(double& c, double& v) {
+    __shared__ double part[2][8];
+    const int t = threadIdx.x, l = t & 31, w = t >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double pc = __shfl_up_sync(0xffffffffu, c, o), pv = __shfl_up_sync(0xffffffffu, v, o);
+        if (l >= o) {
+            c += pc;
+            v += pv;
+        }
+    }
+    __syncthreads();  // part free from a previous call
+    if (l == 31) {
+        part[0][w] = c;
+        part[1][w] = v;
+    }
+    __syncthreads();
+    double bc = 0.0, bv = 0.0;
+    for (int k = 0; k < w; ++k) {
+        bc += part[0][k];
+        bv += part[1][k];
+    }
+    c += bc;
+    v += bv;
 }
 
 // Threshold limiter (Section 4.4), one CTA after every cand_ds entry of the
@@ -1200,94 +1234,112 @@ __device__ __forceinline__ double block_sum(double v) {
 // delta).  With S the step's sum of Delta S over the lattice (partial sums
 // of the step kernel) and R = delta0 (1 - (2 beta - 1)^2) S, the threshold
 // Delta S_0 of Eq. (EntThresh) solves L(t) = sum max(Delta S - t, 0) = R.
-// Only sites above delta matter when L(delta) > R (otherwise Delta S_t =
-// delta); then the sites whose L(Delta S) < R (the "upper" set, n of them
-// with sum S_u) are found by an MSB radix descent over the FP64 bits of the
-// candidate values with per-bin counts and sums, and Delta S_0 =
-// (S_u - R) / n, the root on the linear piece of L below them.  Sites with
-// Delta S >= Delta S_t = max(Delta S_0, delta) get the homothety
+// Only sites above delta matter when L(delta) > R (otherwise, and with R = 0,
+// Delta S_t = delta); then the sites whose L(Delta S) < R (the "upper" set, n
+// of them with sum S_u) give Delta S_0 = (S_u - R) / n, the root on the linear
+// piece of L below them.  Up to 32 candidates (the usual case) one warp takes
+// them, a lane each; more go through an MSB radix descent over the FP64 bits
+// of the candidate values with per-bin counts and sums, a thread per bin.
+// (One thread walking the 256 bins of each digit, three FP64 operations of 64
+// clocks a bin, was 200 us of a step: 2049^2 FP32 272 -> 77 us, 257^2 201 -> 19.)
+// Sites with Delta S >= Delta S_t = max(Delta S_0, delta) get the homothety
 // sqrt(Delta S_t / Delta S) of Eq. (entrHom) before the LBGK collision.
+// CTAs of 256 threads.
 template <int Q, class ST, bool ODD>
 __device__ void threshold_select_apply(const Params& p, unsigned M) {
     using T = typename ST::T;
     __shared__ unsigned cnt[256];
     __shared__ double hsum[256];
     __shared__ unsigned long long s_prefix, s_mask;
-    __shared__ double s_cntA, s_sumA;
-    __shared__ int s_done;
+    __shared__ double s_cntA, s_sumA, s_dst;
+    __shared__ int s_chosen;
     __shared__ unsigned s_count;
     const int tid = threadIdx.x, nt = blockDim.x;
-    // the step's sum of Delta S; the slots are cleared for the next step
-    double S = 0.0;
+    // the step's sum of Delta S (the slots are cleared for the next step) and L(delta)
+    double S = 0.0, Ld = 0.0;
     for (int k = tid; k < kRedSlots; k += nt) {
         S += __ldcg(&p.red[k]);
         p.red[k] = 0.0;
     }
-    S = block_sum(S);
-    const double c = 1.0 - (2.0 * p.beta - 1.0) * (2.0 * p.beta - 1.0);
-    const double R = p.lim_delta0 * c * S;
-    double Ld = 0.0;
     for (unsigned j = tid; j < M; j += nt) {
         const double v = __ldcg(&p.cand_ds[j]);
         if (v > p.delta && v < INFINITY) Ld += v - p.delta;
     }
-    Ld = block_sum(Ld);
+    block_sum2(S, Ld);
+    const double c = 1.0 - (2.0 * p.beta - 1.0) * (2.0 * p.beta - 1.0);
+    const double R = p.lim_delta0 * c * S;
     double dst = p.delta;
     if (Ld > R) {
-        if (tid == 0) {
-            s_prefix = 0ull;
-            s_mask = 0ull;
-            s_cntA = 0.0;
-            s_sumA = 0.0;
-            s_done = 0;
-        }
-        __syncthreads();
-        for (int shift = 56; shift >= 0; shift -= 8) {
-            if (s_done) break;  // uniform: read after the barrier
-            for (int d = tid; d < 256; d += nt) {
-                cnt[d] = 0u;
-                hsum[d] = 0.0;
-            }
-            __syncthreads();
-            const unsigned long long pre = s_prefix, msk = s_mask;
-            for (unsigned j = tid; j < M; j += nt) {
-                const double v = __ldcg(&p.cand_ds[j]);
-                if (!(v > p.delta && v < INFINITY)) continue;
-                const unsigned long long key = (unsigned long long)__double_as_longlong(v);
-                if ((key & msk) != pre) continue;
-                const int d = (int)((key >> shift) & 255ull);
-                atomicAdd(&cnt[d], 1u);
-                atomicAdd(&hsum[d], v);
-            }
-            __syncthreads();
-            if (tid == 0) {
-                // bins from the top: the first whose lower bound b has
-                // L(b) >= R holds the boundary; the bins above it are upper
-                double cA = s_cntA, sA = s_sumA;
-                int chosen = -1;
-                for (int d = 255; d >= 0; --d) {
-                    const double ci = cA + (double)cnt[d], si = sA + hsum[d];
-                    const double b = __longlong_as_double((long long)(pre | ((unsigned long long)d << shift)));
-                    if (si - b * ci >= R) {
-                        chosen = d;
-                        break;
+        if (M <= 32) {
+            if (tid < 32) {
+                double v = (unsigned)tid < M ? __ldcg(&p.cand_ds[tid]) : -1.0;
+                if (!(v > p.delta && v < INFINITY)) v = -1.0;
+                double n = 0.0, su = 0.0;  // count and sum of the values >= v
+                for (unsigned j = 0; j < M; ++j) {
+                    const double o = __shfl_sync(0xffffffffu, v, j);
+                    if (o >= v) {
+                        n += 1.0;
+                        su += o;
                     }
-                    cA = ci;
-                    sA = si;
                 }
-                s_cntA = cA;
-                s_sumA = sA;
-                if (chosen < 0) {
-                    s_done = 1;
-                } else {
-                    s_prefix = pre | ((unsigned long long)chosen << shift);
+                const bool valid = v > 0.0, upper = valid && su - v * n < R;
+                double nu = upper ? 1.0 : 0.0, sum = upper ? v : 0.0;
+                for (int o = 16; o > 0; o >>= 1) {
+                    nu += __shfl_xor_sync(0xffffffffu, nu, o);
+                    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                }
+                if (tid == 0) s_dst = nu > 0.0 ? (sum - R) / nu : p.delta;
+            }
+            __syncthreads();
+        } else {
+            if (tid == 0) {
+                s_prefix = 0ull;
+                s_mask = 0ull;
+                s_cntA = 0.0;
+                s_sumA = 0.0;
+            }
+            for (int shift = 56; shift >= 0; shift -= 8) {
+                cnt[tid] = 0u;
+                hsum[tid] = 0.0;
+                if (tid == 0) s_chosen = 256;
+                __syncthreads();
+                const unsigned long long pre = s_prefix, msk = s_mask;
+                for (unsigned j = tid; j < M; j += nt) {
+                    const double v = __ldcg(&p.cand_ds[j]);
+                    if (!(v > p.delta && v < INFINITY)) continue;
+                    const unsigned long long key = (unsigned long long)__double_as_longlong(v);
+                    if ((key & msk) != pre) continue;
+                    const int d = (int)((key >> shift) & 255ull);
+                    atomicAdd(&cnt[d], 1u);
+                    atomicAdd(&hsum[d], v);
+                }
+                __syncthreads();
+                // bins from the top (thread t: bin 255 - t): the first whose lower
+                // bound b has L(b) >= R holds the boundary; the bins above it are
+                // upper
+                const int d = 255 - tid;
+                const double cA = s_cntA, sA = s_sumA, c0 = (double)cnt[d], h0 = hsum[d];
+                double ci = c0, si = h0;
+                block_scan2(ci, si);
+                ci += cA;
+                si += sA;
+                const double b = __longlong_as_double((long long)(pre | ((unsigned long long)d << shift)));
+                if (si - b * ci >= R) atomicMin(&s_chosen, tid);
+                __syncthreads();
+                const int ch = s_chosen;
+                if (ch == 256 ? tid == 255 : tid == ch) {  // none: every bin is upper
+                    s_cntA = ch == 256 ? ci : ci - c0;
+                    s_sumA = ch == 256 ? si : si - h0;
+                    s_prefix = pre | ((unsigned long long)d << shift);
                     s_mask = msk | (255ull << shift);
                 }
+                __syncthreads();
+                if (ch == 256) break;
             }
+            if (tid == 0) s_dst = s_cntA > 0.0 ? (s_sumA - R) / s_cntA : p.delta;
             __syncthreads();
         }
-        // n = 0: R <= 0 and the boundary is the largest value itself
-        const double t0 = s_cntA > 0.0 ? (s_sumA - R) / s_cntA : __longlong_as_double((long long)s_prefix);
+        const double t0 = s_dst;
         dst = t0 > p.delta ? t0 : p.delta;
     }
     if (tid == 0) s_count = 0u;
@@ -1792,8 +1844,7 @@ __global__ void __launch_bounds__(256) ensemble_mean(Params p) {
         p.red[k] = 0.0;
         p.red[kRedSlots + k] = 0.0;
     }
-    S = block_sum(S);
-    N = block_sum(N);
+    block_sum2(S, N);
     if (t == 0) {
         *p.lim_E = N > 0.0 ? S / N : 0.0;
         *p.lim_E_f = (float)*p.lim_E;
@@ -1815,8 +1866,7 @@ __global__ void __launch_bounds__(256) ensemble_finalize(Params p) {
         p.red[k] = 0.0;
         p.red[kRedSlots + k] = 0.0;
     }
-    S = block_sum(S);
-    N = block_sum(N);
+    block_sum2(S, N);
     if (t == 0) {
         *p.lim_E = N > 0.0 ? S / N : 0.0;
         *p.lim_E_f = (float)*p.lim_E;
