@@ -89,6 +89,13 @@ void fill_params(const lbm_config* cfg, int nsm, Params& p) {
     p.mrt.q = cfg->s_q / 12.0;
     p.mrt.nu = snu / 4.0;
     p.mrt_f = {(float)p.mrt.e, (float)p.mrt.eps, (float)p.mrt.q, (float)p.mrt.nu};
+    {
+        // e = 3 (A + 2 D), eps = -3 (2 A + D); axis rows -e - 2 eps, diagonal rows 2 e + eps
+        const double e = 3.0 * p.mrt.e, ep = -3.0 * p.mrt.eps;
+        p.mrt64 = {-e - 4.0 * ep, -2.0 * (e + ep), 2.0 * (e + ep), 4.0 * e + ep, 3.0 * p.mrt.q, 6.0 * p.mrt.q, p.mrt.nu};
+        p.two_beta = snu;
+        p.mrt2_c = (snu - 1.0) / 4.0;
+    }
     p.elbm_eps = cfg->elbm_eps;
     p.elbm_max_iter = cfg->elbm_max_iter;
     p.elbm_norm = cfg->elbm_norm;

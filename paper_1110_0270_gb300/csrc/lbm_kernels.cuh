@@ -21,6 +21,7 @@
 #pragma once
 
 #include "lbm_elbm_f32.cuh"
+#include "lbm_fp64.cuh"
 
 namespace lbm {
 
@@ -119,6 +120,97 @@ __device__ __forceinline__ void limiter_screen(const Params& p, int x, int y, co
     if (maybe) record_candidate<Q, T>(p, x, y, f);
 }
 
+// The rule on a site with a negative population (out of line: rare).
+static __device__ __noinline__ Pops<9, double> positivity_f64(const Params& p, Pops<9, double> feq, Pops<9, double> F) {
+    if (positivity<9, double>(feq.v, F.v)) atomicAdd(&p.stats[ST_LIMITED], 1ull);
+    return F;
+}
+
+// The collisions of lbm_fp64.cuh on one site.
+template <class ST, int COLL>
+__device__ __forceinline__ void collide_f64(const Params& p, int x, int y, const double* f, double* F) {
+    constexpr bool kScreen = COLL == LBM_EHRENFEST || COLL == LBM_MRT_LIMITER;
+    constexpr bool kRest = kScreen || COLL == LBM_POSITIVITY;  // the rest population's e is needed
+    Eq64 m;
+    double e[9];
+    moments_f64(f, m);
+    if (state_bad(m.rho, m.ux, m.uy))
+        if (*(volatile unsigned*)&p.counters[CNT_DIVERGED] == 0u) atomicExch(&p.counters[CNT_DIVERGED], 1u);
+    if (p.eq != LBM_EQ_POLY_STD) factors_f64(p.eq, m);
+    diff_f64<kRest ? 0 : 1>(p.eq, m, f, e);
+    if (kScreen && screen_f64(p.eq, m, f, e, p.delta_f)) record_candidate<9, double>(p, x, y, f);
+    if (COLL == LBM_MRT)
+        mrt_f64(p.mrt64, f, e, F);
+    else if (COLL == LBM_MRT2)
+        mrt2_f64(p.mrt2_c, f, e, F);
+    else
+        lbgk_f64(p.two_beta, f, e, F);
+    if (COLL == LBM_POSITIVITY) {
+        F[0] = fma(p.two_beta, e[0], f[0]);
+        int sign = 0;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) sign |= __double2hiint(F[i]);
+        if (sign < 0) {
+            Pops<9, double> a, b;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                a.v[i] = f[i] + e[i];
+                b.v[i] = F[i];
+            }
+            b = positivity_f64(p, a, b);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) F[i] = b.v[i];
+        }
+    }
+    mass_f64(m.rho, F);
+}
+
+// The Section 4.2-4.4 limiters on D2Q9 in FP64 (collide_site's arithmetic on
+// the parts of lbm_fp64.cuh): F = f* + (1 - 2 beta) phi (f - f*) =
+// f + (1 - (1 - 2 beta) phi) e.
+template <int Q, class T, int COLL>
+constexpr bool kFp64Lim = Q == 9 && sizeof(T) == 8 &&
+                          ((COLL >= LBM_SMOOTH && COLL <= LBM_THRESHOLD) || COLL == LBM_ENSEMBLE_LAGGED);
+
+template <int COLL>
+__device__ __forceinline__ void collide_lim_f64(const Params& p, int x, int y, const double* f, double* F,
+                                                int& e_code, double& acc) {
+    Eq64 m;
+    double e[9], q;
+    moments_f64(f, m);
+    if (state_bad(m.rho, m.ux, m.uy))
+        if (*(volatile unsigned*)&p.counters[CNT_DIVERGED] == 0u) atomicExch(&p.counters[CNT_DIVERGED], 1u);
+    if (p.eq != LBM_EQ_POLY_STD) factors_f64(p.eq, m);
+    diff_f64<0>(p.eq, m, f, e);
+    const double ds = delta_s_f64(p.eq, m, f, e, q);
+    const bool finite = (__double2hiint(ds) & 0x7ff00000) != 0x7ff00000;
+    double phi = 1.0;
+    if ((COLL == LBM_ENSEMBLE_LAGGED || COLL == LBM_THRESHOLD) && finite) {
+        acc += ds;
+        e_code = 1;
+    }
+    if (COLL == LBM_THRESHOLD) {
+        if (median_maybe_above(finite ? trunc_f32(ds) : INFINITY, trunc_f32(q), trunc_f32(m.rho), p.delta_f))
+            record_candidate<9, double>(p, x, y, f);
+    } else if (!finite) {
+        phi = 0.0;  // a negative population: the state goes to f*
+    } else if (COLL == LBM_SMOOTH) {
+        phi = 1.0 / (1.0 + p.lim_alpha * pow_f64(ds, p.lim_k));
+    } else if (COLL == LBM_DOUBLE_MONOTONIC) {
+        phi = pow_f64(1.0 + pow_f64(ds / p.lim_dst, p.lim_k), -0.5 / p.lim_k);
+    } else {
+        const double E = *p.lim_E;
+        if (E > 0.0) {
+            const double yv = ds / (p.lim_alpha * E);
+            phi = (1.0 + pow_f64(yv, p.lim_k - 0.5)) / (1.0 + pow_f64(yv, p.lim_k));
+        }
+    }
+    const double c = 1.0 - (1.0 - p.two_beta) * phi;
+#pragma unroll
+    for (int i = 1; i < 9; ++i) F[i] = fma(c, e[i], f[i]);
+    mass_f64(m.rho, F);
+}
+
 // Collision of one site, pre-collision f to post-collision F: moments,
 // divergence check, equilibrium, limiter screen, collision, exact mass.
 template <int Q, class ST, int COLL>
@@ -126,6 +218,14 @@ __device__ __forceinline__ void collide_site(const Params& p, int x, int y, cons
                                              typename ST::T* F, int& e_code, int& e_iters,
                                              typename ST::T& acc) {
     using T = typename ST::T;
+    if constexpr (kFp64Form<Q, T, COLL>) {
+        collide_f64<ST, COLL>(p, x, y, f, F);
+        return;
+    }
+    if constexpr (kFp64Lim<Q, T, COLL>) {
+        collide_lim_f64<COLL>(p, x, y, f, F, e_code, acc);
+        return;
+    }
     T rho, ux, uy;
     moments<Q, T>(f, rho, ux, uy);
     // once set the flag is only read: a diverged lattice would otherwise
@@ -858,11 +958,29 @@ constexpr bool kSitePrefetch = Q == 9 && sizeof(typename ST::S) == 4 &&
                                 COLL == LBM_POSITIVITY || COLL == LBM_MRT || COLL == LBM_MRT2 ||
                                 COLL == LBM_MRT_LIMITER || COLL == LBM_SMOOTH);
 
+// D2Q9 in FP64 storage: sites in row-major order, one per thread, in CTAs of
+// kFlatThreads.  The step takes as long as the SM with the most warps (each
+// FP64 instruction costs its SM 19 clocks however few lanes are active), so
+// rows are not padded to whole tiles and the CTAs are small: a 257^2 lattice
+// in 128 x 2 tiles has 387 CTAs for 152 SMs, one in three nearly empty (MRT
+// 42 us a step; 15.3 in CTAs of 256 of this order, 14.9 of 128, 13.7 of 64 or
+// 32; the same at 2049^2).
+template <int Q, class ST>
+constexpr bool kFlat = Q == 9 && sizeof(typename ST::T) == 8;
+constexpr int kFlatThreads = 64;
+
 template <int Q, class ST, int COLL, bool ODD>
 __global__ void __launch_bounds__(kBlockX* kBlockY, kMinBlocks<ST, COLL>) step_kernel(Params p) {
     pdl_enter();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int x, y;
+    if constexpr (kFlat<Q, ST>) {
+        const unsigned s = blockIdx.x * blockDim.x + threadIdx.x;
+        y = (int)(s / (unsigned)p.nx);
+        x = (int)(s - (unsigned)y * (unsigned)p.nx);
+    } else {
+        x = blockIdx.x * blockDim.x + threadIdx.x;
+        y = blockIdx.y * blockDim.y + threadIdx.y;
+    }
     constexpr bool kLimiter =
         (COLL == LBM_EHRENFEST || COLL == LBM_MEDIAN || COLL == LBM_THRESHOLD || COLL == LBM_MRT_LIMITER);
     if (kLimiter && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
@@ -1820,6 +1938,12 @@ __global__ void __launch_bounds__(256) ensemble_mean(Params p) {
             // the Delta S the step's collision computes (collide_lim)
             lim_state(p.eq, f, rho, ux, uy, feq);
             ds = delta_s_lim(f, feq, q);
+        } else if constexpr (kFp64Lim<Q, T, LBM_ENSEMBLE>) {
+            Eq64 m;
+            moments_f64(f, m);
+            if (p.eq != LBM_EQ_POLY_STD) factors_f64(p.eq, m);
+            diff_f64<0>(p.eq, m, f, feq);
+            ds = delta_s_f64(p.eq, m, f, feq, q);
         } else {
             moments<Q, T>(f, rho, ux, uy);
             equilibrium<Q, T>(p.eq, rho, ux, uy, feq);
@@ -2424,7 +2548,11 @@ cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
         int t = ((p.nx + nsm - 1) / nsm + 31) / 32 * 32;
         b = dim3(t < 32 ? 32 : (t > 256 ? 256 : t), 1);
     }
-    const dim3 g = site_grid(p, b);
+    dim3 g = site_grid(p, b);
+    if (kFlat<Q, ST>) {
+        b = dim3(kFlatThreads);
+        g = dim3((unsigned)(((int64_t)p.nx * p.ny + kFlatThreads - 1) / kFlatThreads));
+    }
     return launch_p(odd ? step_kernel<Q, ST, COLL, true> : step_kernel<Q, ST, COLL, false>, g, b, s, p);
 }
 

@@ -15,6 +15,11 @@ struct MrtRates {
 struct MrtRatesF {
     float e, eps, q, nu;
 };
+// The coefficients of mrt_f64: axis and diagonal even parts from the sums over
+// the axis (A) and diagonal (D) populations, q_x and q_y rows, p_xx and p_xy.
+struct Mrt64 {
+    double aA, aD, dA, dD, q, q2, nu;
+};
 
 // Device counters (one 256-byte block of scratch, zeroed at create).
 enum Counter {
@@ -59,6 +64,8 @@ struct Params {
     double delta;
     MrtRates mrt;
     MrtRatesF mrt_f;
+    Mrt64 mrt64;
+    double two_beta, mrt2_c;         // 2 beta, (2 beta - 1) / 4 (no per-site FP64 arithmetic)
     double elbm_eps;
     int elbm_max_iter, elbm_norm, elbm_fallback;
     double elbm_skip_rel;  // near-equilibrium skip: Delta S < 1e-15 + elbm_skip_rel * rho
