@@ -3,6 +3,7 @@
 // into the population array and the scratch the limiters need.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -362,6 +363,37 @@ cudaError_t capture_periods(lbm_ctx* ctx, int periods, cudaGraph_t* graph, cudaG
     return e;
 }
 
+// The steps of this context that line_steps takes: a D1Q3 line of a collision
+// local to the site, in FP64 or FP32 (ELBM: FP32), no probe (sampled every
+// step) and no per-kernel timing.
+bool line_form(const lbm_ctx* ctx, int& threads, int& halo) {
+    const int coll = ctx->cfg.collision, prec = ctx->cfg.precision;
+    if (ctx->Q != 3 || ctx->profiling || ctx->p.probe_buf) return false;
+    if (prec != LBM_FP64 && prec != LBM_FP32) return false;
+    if (coll != LBM_LBGK && coll != LBM_MRT && coll != LBM_SMOOTH && coll != LBM_DOUBLE_MONOTONIC &&
+        !(coll == LBM_ELBM && prec == LBM_FP32))
+        return false;
+    return line_window(ctx->cfg.nx, ctx->nsm, threads, halo);
+}
+
+// n (even, >= 2) steps from an even step count: pairs of launches through the
+// staging area (3 nx doubles, otherwise scratch of lbm_init and lbm_enstrophy) and back.
+cudaError_t enqueue_line(lbm_ctx* ctx, int n, int threads, int halo, cudaStream_t s) {
+    const Params& p = ctx->p;
+    for (int k = 0; k < n;) {
+        const int m = std::min(n - k, 2 * halo), a = m / 2, b = m - a;
+        cudaError_t e = dispatch(ctx->cfg.precision, [&](auto L) {
+            cudaError_t r = decltype(L)::line(ctx->cfg.collision, p, p.f, p.plane, ctx->staging, p.nx, threads, a, halo, s);
+            return r != cudaSuccess ? r
+                                    : decltype(L)::line(ctx->cfg.collision, p, ctx->staging, p.nx, p.f, p.plane, threads,
+                                                        b, halo, s);
+        });
+        if (e != cudaSuccess) return e;
+        k += m;
+    }
+    return cudaSuccess;
+}
+
 // The two-step graph lbm_step replays, and for long runs of small lattices
 // (where the host's graph launches, not the GPU, set the pace) one of
 // kLongPeriods periods.
@@ -579,7 +611,19 @@ lbm_status lbm_step(lbm_ctx* ctx, int nsteps, void* stream) {
     if (nsteps < 0) return fail(ctx, LBM_ERR_ARG, "nsteps must be >= 0");
     // parity == t & 1 always (both reset together), so the graph, whose
     // steps use counter slots 0 and 1, starts at an even step
-    int k = 0;
+    int k = 0, threads = 0, halo = 0;
+    if (ctx->parity == 1 && nsteps > 2 && line_form(ctx, threads, halo)) {
+        LBM_CK(ctx, enqueue_one_step(ctx, true, 1, S(stream)));
+        ctx->parity = 0;
+        ctx->t += 1;
+        k = 1;
+    }
+    if (ctx->parity == 0 && nsteps - k >= 2 && line_form(ctx, threads, halo)) {
+        const int n = (nsteps - k) & ~1;
+        LBM_CK(ctx, enqueue_line(ctx, n, threads, halo, S(stream)));
+        ctx->t += n;
+        k += n;
+    }
     const bool use_graph = ctx->graph_exec && !ctx->profiling;
     while (k < nsteps) {
         if (use_graph && ctx->parity == 0 && ctx->graph_long_exec && nsteps - k >= 2 * kLongPeriods) {

@@ -1000,6 +1000,99 @@ __global__ void __launch_bounds__(kBlockX* kBlockY, kMinBlocks<ST, COLL>) step_k
         block_sum_to_slots<typename ST::T>(p, acc, e_code == 1 ? typename ST::T(1) : typename ST::T(0), true);
 }
 
+// Several steps of a D1Q3 line in one launch, for the collisions that need
+// nothing but the site itself.  A step of a few hundred sites is one launch
+// (2 us) for a chain of a third of that, so each CTA carries a window of the
+// line through `steps` steps in registers: neighbours' populations come by
+// shuffle (across warps by shared memory), and a halo of `halo` >= steps sites
+// on either side, computed again by the neighbouring CTA, loses one site a
+// step.  Natural layout on both sides (f_i(x) at i * plane + x, what an even
+// step count leaves in place), src and dst distinct: two launches return the
+// state to its buffer.  A site is computed as step_kernel computes it; FP64
+// and FP32 storage only, whose populations lose nothing between steps.
+// 800-site tube, LBGK FP64: 2.36 us a step -> 0.97 (400 steps and their set-up 0.93 -> 0.40 ms).
+template <class ST, int COLL>
+constexpr bool kLineForm = sizeof(typename ST::S) == sizeof(typename ST::T) &&
+                           (COLL == LBM_LBGK || COLL == LBM_MRT || COLL == LBM_SMOOTH ||
+                            COLL == LBM_DOUBLE_MONOTONIC || kElbmWarp<ST, COLL>);
+constexpr int kLineThreads = 256;
+
+template <class ST, int COLL>
+__global__ void __launch_bounds__(kLineThreads) line_steps(Params p, const void* src_, int64_t sp, void* dst_,
+                                                           int64_t dp, int steps, int halo) {
+    pdl_enter();
+    using T = typename ST::T;
+    __shared__ T edge[2][2][kLineThreads / 32];  // by step parity: F_2 of a warp's last site, F_0 of its first
+    const T* src = (const T*)src_;
+    const int t = threadIdx.x, n = blockDim.x, lane = t & 31, w = t >> 5;
+    const int x = (int)blockIdx.x * (n - 2 * halo) - halo + t;
+    const bool own = t >= halo && t < n - halo && x < p.nx;
+    int xs = x;
+    bool valid = x >= 0 && x < p.nx;
+    if (p.periodic_x) {
+        xs = x % p.nx;
+        if (xs < 0) xs += p.nx;
+        valid = true;
+    }
+    const bool first = !p.periodic_x && x == 0, last = !p.periodic_x && x == p.nx - 1;
+    T f[3] = {T(1), T(1), T(1)};
+    if (valid) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) f[i] = src[i * sp + xs];
+    }
+    for (int s = 0; s < steps; ++s) {
+        T F[3] = {f[0], f[1], f[2]}, acc = T(0);
+        int e_code = -1, e_iters = 0;
+        // the sites whose state is still the line's own
+        const bool on = valid && t >= s && t < n - s;
+        if constexpr (kElbmWarp<ST, COLL>) {
+            T G[3];
+            elbm_warp<3>(p, on, f, G, e_code, e_iters);
+            if (on) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) F[i] = G[i];
+            }
+            elbm_stats(p, own ? e_code : -1, own ? e_iters : 0);
+        } else if (on) {
+            collide_site<3, ST, COLL>(p, xs, 0, f, F, e_code, e_iters, acc);
+        }
+        // F_0 moves left, F_2 right; at a wall the population comes back
+        T l = __shfl_down_sync(0xffffffffu, F[0], 1), r = __shfl_up_sync(0xffffffffu, F[2], 1);
+        if (n > 32) {
+            if (lane == 31) edge[s & 1][0][w] = F[2];
+            if (lane == 0) edge[s & 1][1][w] = F[0];
+            __syncthreads();
+            if (lane == 31 && t + 1 < n) l = edge[s & 1][1][w + 1];
+            if (lane == 0 && w > 0) r = edge[s & 1][0][w - 1];
+        }
+        f[0] = last ? F[2] : l;
+        f[1] = F[1];
+        f[2] = first ? F[0] : r;
+    }
+    if (own) {
+        T* dst = (T*)dst_;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) dst[i * dp + x] = f[i];
+    }
+}
+
+// The window of line_steps: the fewest warps whose CTAs, one per SM, cover the
+// line with a halo of at least six sites (one warp) or eight, and the widest
+// halo up to twelve that then fits.  Longer lines (above 240 sites an SM) keep
+// a launch per step: there the arithmetic, not the launch, sets the time.
+inline bool line_window(int nx, int nsm, int& threads, int& halo) {
+    const int own = (nx + nsm - 1) / nsm;
+    for (int w = 1; w <= kLineThreads / 32; ++w) {
+        int h = (32 * w - own) / 2;
+        if (h > 12) h = 12;
+        if (h < (w == 1 ? 6 : 8)) continue;
+        threads = 32 * w;
+        halo = h;
+        return true;
+    }
+    return false;
+}
+
 // ELBM on a D1Q3 line in FP64 storage, four lanes per site (elbm_lanes): lane
 // q < 3 of a group owns population q, its address included.  CTAs of one
 // warp (eight sites), so that a line of a few hundred sites spreads over the
@@ -2457,6 +2550,8 @@ __global__ void __launch_bounds__(256) entropy_kernel(Params p, double* H, doubl
 template <class ST>
 struct Launch {
     static cudaError_t step(int Q, int coll, bool odd, const Params& p, cudaStream_t s);
+    static cudaError_t line(int coll, const Params& p, const void* src, int64_t sp, void* dst, int64_t dp, int threads,
+                            int steps, int halo, cudaStream_t s);
     static cudaError_t fixup(int Q, int coll, bool odd, const Params& p, cudaStream_t s, int nsm);
     static cudaError_t prepass(int Q, int coll, bool odd, const Params& p, cudaStream_t s);
     static cudaError_t probe(int Q, bool odd, const Params& p, cudaStream_t s);
@@ -2474,6 +2569,22 @@ struct Launch {
                                cudaStream_t s);
     static cudaError_t cand_eval(int Q, const Params& p, unsigned n, cudaStream_t s);
 };
+
+// Launch with programmatic dependence on the stream's previous kernel (the
+// kernel starts with pdl_enter).
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*k)(P...), dim3 g, dim3 b, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = g;
+    c.blockDim = b;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, args...);
+}
 
 inline cudaError_t launch_p(void (*k)(Params, int), dim3 g, dim3 b, cudaStream_t s, const Params& p, int a) {
     if (!p.pdl) {
@@ -2620,6 +2731,30 @@ cudaError_t launch_prepass_q(int coll, bool odd, const Params& p, cudaStream_t s
 template <class ST>
 cudaError_t Launch<ST>::step(int Q, int coll, bool odd, const Params& p, cudaStream_t s) {
     return Q == 3 ? launch_step_c<3, ST>(coll, odd, p, s) : launch_step_c<9, ST>(coll, odd, p, s);
+}
+
+template <class ST, int COLL>
+cudaError_t launch_line(const Params& p, const void* src, int64_t sp, void* dst, int64_t dp, int threads, int steps,
+                        int halo, cudaStream_t s) {
+    if constexpr (kLineForm<ST, COLL>) {
+        const int own = threads - 2 * halo;
+        return launch_pdl(line_steps<ST, COLL>, (p.nx + own - 1) / own, threads, s, p, src, sp, dst, dp, steps, halo);
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <class ST>
+cudaError_t Launch<ST>::line(int coll, const Params& p, const void* src, int64_t sp, void* dst, int64_t dp,
+                             int threads, int steps, int halo, cudaStream_t s) {
+    switch (coll) {
+        case LBM_LBGK: return launch_line<ST, LBM_LBGK>(p, src, sp, dst, dp, threads, steps, halo, s);
+        case LBM_MRT: return launch_line<ST, LBM_MRT>(p, src, sp, dst, dp, threads, steps, halo, s);
+        case LBM_SMOOTH: return launch_line<ST, LBM_SMOOTH>(p, src, sp, dst, dp, threads, steps, halo, s);
+        case LBM_DOUBLE_MONOTONIC:
+            return launch_line<ST, LBM_DOUBLE_MONOTONIC>(p, src, sp, dst, dp, threads, steps, halo, s);
+        case LBM_ELBM: return launch_line<ST, LBM_ELBM>(p, src, sp, dst, dp, threads, steps, halo, s);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <class ST>
