@@ -9,7 +9,7 @@
 // and divisions run side by side, and only their sums cross lanes.
 #pragma once
 
-#include "lbm_device.cuh"
+#include "lbm_fp64.cuh"
 
 namespace lbm {
 
@@ -35,26 +35,76 @@ __device__ __forceinline__ float warp_max(float v) {  // v >= 0
     return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
 }
 
+// sum_k c[k] z^k, K coefficients by pairs (Estrin): a chain of log2 K steps
+// instead of K.  c is overwritten.
+template <int K>
+__device__ __forceinline__ double estrin(double* c, double z) {
+#pragma unroll
+    for (int n = K; n > 1; n = (n + 1) / 2) {
+#pragma unroll
+        for (int k = 0; k < n / 2; ++k) c[k] = fma(c[2 * k + 1], z, c[2 * k]);
+        if (n & 1) c[n / 2] = c[n - 1];
+        z *= z;
+    }
+    return c[0];
+}
+// gl_series<KG, KL> with its series by pairs.
+template <int KG, int KL>
+__device__ __forceinline__ void gl_pairs(double x, double& g, double& l) {
+    constexpr int K = KL > KG + 1 ? KL : KG + 1;
+    double c[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) c[j] = ((j & 1) ? 1.0 : -1.0) / (double)(j + 2);
+    const double m = x * estrin<K>(c, x);
+    l = fma(x, m, x);
+    g = x * fma(m, 1.0 + x, x);
+}
+// g(x) and ln(1 + x) by the area tangent series: with s = x / (2 + x),
+// ln(1 + x) = 2 artanh s = 2 s (1 + s^2 R), R = sum_{k<K} s^2k / (2k + 3), and
+// from x = 2 s / (1 - s), g(x) = x s (1 + s R (1 + s)): no cancellation in
+// either.  Converges like (x / 2)^2k where the Taylor series has x^k: 9 terms
+// for |x| < 1/4 (27), 17 for 1/2.  The first omitted term is below 2^-56 of
+// the leading one.  |x| <= 1/2 (2 + x: no range check on its reciprocal).
+template <int K>
+__device__ __forceinline__ void gl_artanh(double x, double& g, double& l) {
+    float seed;
+    const double y = 2.0 + x;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(seed) : "f"(trunc_f32(y)));
+    const double r = widen_f64(seed), e = fma(-y, r, 1.0);
+    const double s = x * fma(r, fma(e, e, e), r);  // x / (2 + x), as in rcp_f64
+    double c[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) c[k] = 1.0 / (double)(2 * k + 3);
+    const double w = s * estrin<K>(c, s * s), s2 = s + s;
+    l = fma(s2 * s, w, s2);
+    g = (x * s) * fma(w, 1.0 + s, 1.0);
+}
+
 // g(x) and ln(1 + x) at one population; am >= |x| over the warp picks the
-// series length (elbm_eval's tiers), so that the lanes take one branch.
+// series length, so that the lanes take one branch.  The sites next to a
+// shock (|x| to 1/2) set the step's time, since it lasts as long as its
+// longest chain: a Horner chain of 27 terms and log1p there made the 800-site
+// tube 20.6 us a step (now 15.6).
 __device__ __forceinline__ void gl_lane(double x, float am, double& g, double& l) {
     if (am < 0x1p-20f)
         gl_series<2, 2>(x, g, l);
     else if (am < 0x1p-10f)
-        gl_series<5, 5>(x, g, l);
+        gl_pairs<5, 5>(x, g, l);
     else if (am < 0.015625f)
-        gl_series<8, 9>(x, g, l);
+        gl_pairs<8, 9>(x, g, l);
     else if (am < 0.125f)
-        gl_series<16, 18>(x, g, l);
+        gl_artanh<7>(x, g, l);
     else if (am < 0.25f)
-        gl_series<26, 27>(x, g, l);
+        gl_artanh<9>(x, g, l);
+    else if (am < 0.5f)
+        gl_artanh<17>(x, g, l);
     else {
         const double xc = x < -1.0 ? -1.0 : x;
         l = log1p(xc);
         g = xc <= -1.0 ? 1.0 : (1.0 + xc) * l - xc;
         if (fabs(x) < 0.25) {  // the closed form cancels for the small ones
             double gs, ls;
-            gl_series<26, 27>(x, gs, ls);
+            gl_artanh<9>(x, gs, ls);
             g = gs;
         }
     }
@@ -97,14 +147,14 @@ __device__ ElbmLane elbm_lanes(const Params& p, double f, bool valid) {
     const double r = group_sum<G>(f);
     const double jx = group_sum<G>(cx > 0 ? f : (cx < 0 ? -f : 0.0));
     const double jy = Q == 9 ? group_sum<G>(cy > 0 ? f : (cy < 0 ? -f : 0.0)) : 0.0;
-    const double ri = 1.0 / (valid ? r : 1.0);
+    const double ri = rcp_f64(valid ? r : 1.0);
     const double ux = jx * ri, uy = jy * ri;
     o.rho = r;
     o.ux = ux;
     o.uy = uy;
     // 1D factors: the lower half of a D2Q9 group works on x, the upper on y
     double u = Q == 9 && (q & 8) ? uy : ux;
-    const double a = (2.0 * sqrt(1.0 + 3.0 * u * u) - 1.0) * (1.0 / 6.0);
+    const double a = fma(sqrt_f64(fma(3.0 * u, u, 1.0)), 1.0 / 3.0, -1.0 / 6.0);
     const int base = lane & ~(G - 1);
     const double aX = Q == 9 ? __shfl_sync(0xffffffffu, a, base) : a;
     const double fX = cx == 0 ? 1.0 - 2.0 * aX : aX + (0.5 * cx) * ux;
@@ -114,7 +164,7 @@ __device__ ElbmLane elbm_lanes(const Params& p, double f, bool valid) {
         fe *= cy == 0 ? 1.0 - 2.0 * aY : aY + (0.5 * cy) * uy;
     }
     const double D = act ? fe - f : 0.0;
-    const double d = act ? D / fe : 0.0;
+    const double d = act ? D * rcp_f64(fe) : 0.0;
     o.D = D;
     const float Df = (float)D, df = (float)d, fef = (float)fe, ff = (float)f;
     const float dmax = group_max<G>(fabsf(df));
@@ -133,7 +183,7 @@ __device__ ElbmLane elbm_lanes(const Params& p, double f, bool valid) {
         mb = t > mb ? t : mb;
     }
     const double rneg = __longlong_as_double(mb);
-    const double amax = mb ? 1.0 + 1.0 / rneg : __longlong_as_double(0x7ff0000000000000ULL);
+    const double amax = mb ? 1.0 + rcp_f64(rneg) : __longlong_as_double(0x7ff0000000000000ULL);
     const double fb = p.elbm_fallback == LBM_FALLBACK_EHRENFEST ? 1.0 : amax;
     o.code = 0;
     o.alpha = 2.0;
@@ -227,7 +277,7 @@ __device__ ElbmLane elbm_lanes(const Params& p, double f, bool valid) {
         // the greater root of the parabola: where S_f falls (s1 < 0) it is
         // t 2 / (1 + sqrt(1 - e)) with t = -s0 / s1, e = 2 s0 s2 / s1^2: t and
         // a correction that FP32 holds to 1e-7 of itself
-        const double t = -s0 / s1;
+        const double t = s0 * rcp_f64(-s1);
         const float e = -2.f * (float)t * s2 / (float)s1;
         const float w = 1.f + sqrtf(1.f - e);
         double next = fma(t, (double)__fdividef(e, w * w), al + t);
@@ -252,7 +302,7 @@ __device__ ElbmLane elbm_lanes(const Params& p, double f, bool valid) {
                 hi = al;
         }
     }
-    if (!done) o.alpha = s0 < 0.0 ? al - 2.0 * s0 / s1 : al;
+    if (!done) o.alpha = s0 < 0.0 ? fma(2.0 * s0, rcp_f64(-s1), al) : al;
     return o;
 }
 
