@@ -321,11 +321,9 @@ cudaError_t enqueue_one_step(lbm_ctx* ctx, bool odd, int cslot, cudaStream_t s) 
         });
     if (e == cudaSuccess)
         e = traced(ctx, LBM_KERNEL_STEP, s, [&] {
-            return dispatch(ctx->cfg.precision,
+            return dispatch(ctx->cfg.precision,  // diffusive wall sites included
                             [&](auto L) { return decltype(L)::step(ctx->Q, coll, odd, q, s); });
         });
-    if (e == cudaSuccess && q.diffusive)  // the wall sites of the same step
-        e = dispatch(ctx->cfg.precision, [&](auto L) { return decltype(L)::walls(odd, q, s); });
     if (e == cudaSuccess && (limiter(coll) || coll == LBM_ENSEMBLE_LAGGED))
         e = traced(ctx, LBM_KERNEL_FIXUP, s, [&] {
             return dispatch(ctx->cfg.precision,

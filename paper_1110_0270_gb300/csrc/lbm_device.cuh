@@ -962,20 +962,79 @@ __device__ __forceinline__ void store_interior(const Params& p, int o, const typ
         ST::st(base + interior_offset<Q, ST, ODD>(p, o, i), F[L::opp(i)], DEV ? T(0) : T(L::w(i)));
 }
 
-// Boundary (or any) site: the general addressing with wrap-around and walls,
-// one direction at a time so that no address array stays live.
+// Boundary (or any) site: the general addressing with wrap-around and walls
+// (aa_address's, which it equals for every direction), by selects, so that the
+// nine loads go out together.  With a branch per direction each load waited
+// for the one before: an odd step's warps with an edge site took nine L2
+// latencies in a row, and on a 129^2 to 513^2 lattice a quarter or more of the
+// warps has one (257^2 MRT in FP64: 13.8 -> 12.8 us a step).
 // (W_i = W_opp(i), so the deviation formats need no slot bookkeeping.)
+template <int Q, class T>
+struct OddGeo {
+    int xs[3], ys[3];      // source column, source row's offset, by v_x + 1, v_y + 1
+    bool okx[3], oky[3];   // inside the domain
+    int o;                 // the site's own offset
+    bool top;              // links of v_y = -1 come from above the top row
+
+    __device__ __forceinline__ OddGeo(const Params& p, int x, int y) {
+        o = y * p.pitch + x;
+        xs[1] = x;
+        okx[1] = oky[1] = true;
+        // source column of v_x = +1: x - 1; of v_x = -1: x + 1
+        xs[2] = x - 1;
+        xs[0] = x + 1;
+        if (p.periodic_x) {
+            xs[2] = xs[2] < 0 ? xs[2] + p.nx : xs[2];
+            xs[0] = xs[0] >= p.nx ? xs[0] - p.nx : xs[0];
+        }
+        okx[2] = xs[2] >= 0;
+        okx[0] = xs[0] < p.nx;
+        ys[1] = y * p.pitch;
+        int yd = y - 1, yu = y + 1;  // sources of v_y = +1, -1
+        if (Q == 9 && p.periodic_y) {
+            yd = yd < 0 ? yd + p.ny : yd;
+            yu = yu >= p.ny ? yu - p.ny : yu;
+        }
+        oky[2] = yd >= 0;
+        oky[0] = yu < p.ny;
+        ys[2] = yd * p.pitch;
+        ys[0] = yu * p.pitch;
+        top = Q == 9 && y + 1 >= p.ny;
+    }
+    // element offset of direction i
+    __device__ __forceinline__ int at(const Params& p, int i) const {
+        using L = Lat<Q>;
+        const int a = L::cx(i) + 1, b = L::cy(i) + 1;
+        return okx[a] && oky[b] ? L::opp(i) * p.plane32 + ys[b] + xs[a] : i * p.plane32 + o;
+    }
+    // the lid term of direction i (v_y = -1 only)
+    __device__ __forceinline__ T lid(const Params& p, int i) const {
+        using L = Lat<Q>;
+        const int a = L::cx(i) + 1, b = L::cy(i) + 1;
+        const int j = L::opp(i);
+        return top && !(okx[a] && oky[b])
+                   ? T(6.0 * L::w(j) * L::cx(j)) * (sizeof(T) == 8 ? T(p.lid_u) : T(p.lid_u_f))
+                   : T(0);
+    }
+};
+
 template <int Q, class ST, bool ODD, bool DEV = false>
 __device__ __forceinline__ void load_general(const Params& p, int x, int y, typename ST::T* f) {
     using T = typename ST::T;
     using L = Lat<Q>;
     const typename ST::S* base = (const typename ST::S*)p.f;
+    if (!ODD) {
+        const int o = y * p.pitch + x;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        T lidc;
-        const int64_t r = aa_address<Q, T>(p, x, y, i, ODD, lidc);
-        f[i] = ST::ld(base + r, DEV ? T(0) : T(L::w(i))) - lidc;
+        for (int i = 0; i < Q; ++i) f[i] = ST::ld(base + i * p.plane32 + o, DEV ? T(0) : T(L::w(i)));
+        return;
     }
+    const OddGeo<Q, T> g(p, x, y);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) f[i] = ST::ld(base + g.at(p, i), DEV ? T(0) : T(L::w(i)));
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+        if (L::cy(i) < 0 && L::cx(i) != 0) f[i] -= g.lid(p, i);
 }
 
 template <int Q, class ST, bool ODD, bool DEV = false>
@@ -984,11 +1043,17 @@ __device__ __forceinline__ void store_general(const Params& p, int x, int y,
     using T = typename ST::T;
     using L = Lat<Q>;
     typename ST::S* base = (typename ST::S*)p.f;
+    if (!ODD) {
+        const int o = y * p.pitch + x;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) ST::st(base + i * p.plane32 + o, F[L::opp(i)], DEV ? T(0) : T(L::w(i)));
+        return;
+    }
+    const OddGeo<Q, T> g(p, x, y);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        T lidc;
-        const int64_t r = aa_address<Q, T>(p, x, y, i, ODD, lidc);
-        ST::st(base + r, F[L::opp(i)] - lidc, DEV ? T(0) : T(L::w(i)));
+        const T v = L::cy(i) < 0 && L::cx(i) != 0 ? F[L::opp(i)] - g.lid(p, i) : F[L::opp(i)];
+        ST::st(base + g.at(p, i), v, DEV ? T(0) : T(L::w(i)));
     }
 }
 

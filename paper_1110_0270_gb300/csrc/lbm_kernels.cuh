@@ -765,6 +765,37 @@ __device__ __forceinline__ void diffusive_rule(const Params& p, int x, int y, T*
         if (L::cx(i) * nxw + L::cy(i) * nyw < 0) f[i] = gamma * feq[i];
 }
 
+// Diffusive Maxwell walls (Section 8): wall site k of one step - load
+// (streaming), the rule of diffusive_rule, store without collision.  k walks
+// the perimeter: bottom row, top row, then the two side columns.
+__host__ __device__ inline int wall_sites(const Params& p) { return 2 * p.nx + 2 * (p.ny - 2); }
+
+template <class ST, bool ODD>
+__device__ __forceinline__ void wall_site(const Params& p, int k) {
+    using T = typename ST::T;
+    const int side = p.ny - 2;
+    int x, y;
+    if (k < p.nx) {
+        x = k;
+        y = 0;
+    } else if (k < 2 * p.nx) {
+        x = k - p.nx;
+        y = p.ny - 1;
+    } else if (k < 2 * p.nx + side) {
+        x = 0;
+        y = 1 + (k - 2 * p.nx);
+    } else if (k < 2 * p.nx + 2 * side) {
+        x = p.nx - 1;
+        y = 1 + (k - 2 * p.nx - side);
+    } else {
+        return;
+    }
+    T f[9];
+    load_general<9, ST, ODD>(p, x, y, f);
+    diffusive_rule<T>(p, x, y, f);
+    store_general<9, ST, ODD>(p, x, y, f);
+}
+
 // The whole step for the site (x, y): load (streaming in odd steps),
 // collision, store.
 // The 16-bit D2Q9 collisions that run in deviation form (collide_dev),
@@ -790,14 +821,16 @@ __device__ __forceinline__ void site_update(const Params& p, int x, int y, int& 
     T f[Q], F[Q];
     const bool interior = x > 0 && x < p.nx - 1 && (Q == 3 || (y > 0 && y < p.ny - 1));
     const int o = y * p.pitch + x;
-    if (interior) {
+    // diffusive walls: wall sites are updated by wall_site (each site owns its
+    // addresses, so the order does not matter)
+    if (Q == 9 && p.diffusive && !interior) return;
+    // a warp with an edge site takes the general addressing for all its sites:
+    // both forms one after the other would take two memory latencies
+    const bool fast = __all_sync(__activemask(), interior);
+    if (fast)
         load_interior<Q, ST, ODD, DEV>(p, o, f);
-    } else {
-        // diffusive walls: wall sites are updated by diffusive_wall_kernel
-        // (each site owns its addresses, so the two kernels of a step commute)
-        if (Q == 9 && p.diffusive) return;
+    else
         load_general<Q, ST, ODD, DEV>(p, x, y, f);
-    }
     if constexpr (DEV) {
         collide_dev<float, ST, COLL>(p, x, y, f, F);
     } else if constexpr (kLimForm<Q, ST, COLL>) {
@@ -809,7 +842,7 @@ __device__ __forceinline__ void site_update(const Params& p, int x, int y, int& 
     } else {
         collide_site<Q, ST, COLL>(p, x, y, f, F, e_code, e_iters, acc);
     }
-    if (interior)
+    if (fast)
         store_interior<Q, ST, ODD, DEV>(p, o, F);
     else
         store_general<Q, ST, ODD, DEV>(p, x, y, F);
@@ -825,16 +858,17 @@ __device__ __forceinline__ void elbm_update(const Params& p, int x, int y, bool 
     float f[Q], F[Q];
     const bool interior = x > 0 && x < p.nx - 1 && (Q == 3 || (y > 0 && y < p.ny - 1));
     const int o = y * p.pitch + x;
-    if (Q == 9 && p.diffusive && !interior) valid = false;  // diffusive_wall_kernel's sites
+    if (Q == 9 && p.diffusive && !interior) valid = false;  // wall_site's
+    const bool fast = __all_sync(0xffffffffu, interior || !valid);
     if (valid) {
-        if (interior)
+        if (fast)
             load_interior<Q, ST, ODD>(p, o, f);
         else
             load_general<Q, ST, ODD>(p, x, y, f);
     }
     elbm_warp<Q>(p, valid, f, F, e_code, e_iters);
     if (valid) {
-        if (interior)
+        if (fast)
             store_interior<Q, ST, ODD>(p, o, F);
         else
             store_general<Q, ST, ODD>(p, x, y, F);
@@ -969,17 +1003,35 @@ template <int Q, class ST>
 constexpr bool kFlat = Q == 9 && sizeof(typename ST::T) == 8;
 constexpr int kFlatThreads = 64;
 
-template <int Q, class ST, int COLL, bool ODD>
+// WALLS (diffusive walls): the CTAs behind the lattice's own take the wall
+// sites, beside the collisions instead of in a kernel after them (6 us
+// of a 28 us step of the 100^2 box in FP64).
+template <int Q, class ST, int COLL, bool ODD, bool WALLS = false>
 __global__ void __launch_bounds__(kBlockX* kBlockY, kMinBlocks<ST, COLL>) step_kernel(Params p) {
     pdl_enter();
     int x, y;
     if constexpr (kFlat<Q, ST>) {
         const unsigned s = blockIdx.x * blockDim.x + threadIdx.x;
+        if constexpr (WALLS) {
+            const unsigned b = (unsigned)(p.nx * p.ny + kFlatThreads - 1) / kFlatThreads;
+            if (blockIdx.x >= b) {
+                wall_site<ST, ODD>(p, (int)(s - b * kFlatThreads));
+                return;
+            }
+        }
         y = (int)(s / (unsigned)p.nx);
         x = (int)(s - (unsigned)y * (unsigned)p.nx);
     } else {
         x = blockIdx.x * blockDim.x + threadIdx.x;
         y = blockIdx.y * blockDim.y + threadIdx.y;
+        if constexpr (WALLS) {
+            const unsigned b = (unsigned)(p.ny + kBlockY - 1) / kBlockY;
+            if (blockIdx.y >= b) {
+                wall_site<ST, ODD>(p, ((blockIdx.y - b) * gridDim.x + blockIdx.x) * (kBlockX * kBlockY) +
+                                          threadIdx.y * kBlockX + threadIdx.x);
+                return;
+            }
+        }
     }
     constexpr bool kLimiter =
         (COLL == LBM_EHRENFEST || COLL == LBM_MEDIAN || COLL == LBM_THRESHOLD || COLL == LBM_MRT_LIMITER);
@@ -2419,35 +2471,12 @@ __global__ void get_state_kernel(Params p, Out* dst, int odd) {
     for (int i = 0; i < Q; ++i) dst[i * N + s] = (Out)f[i];
 }
 
-// Diffusive Maxwell walls (Section 8): the wall sites of one step - load
-// (streaming), the rule of diffusive_rule, store without collision.  Thread
-// k walks the perimeter: bottom row, top row, then the two side columns.
+// The wall sites of one step in a kernel of their own (after the 16-bit pair
+// kernel; step_kernel carries them itself).
 template <class ST, bool ODD>
 __global__ void __launch_bounds__(256) diffusive_wall_kernel(Params p) {
     pdl_enter();
-    using T = typename ST::T;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int side = p.ny - 2;
-    int x, y;
-    if (k < p.nx) {
-        x = k;
-        y = 0;
-    } else if (k < 2 * p.nx) {
-        x = k - p.nx;
-        y = p.ny - 1;
-    } else if (k < 2 * p.nx + side) {
-        x = 0;
-        y = 1 + (k - 2 * p.nx);
-    } else if (k < 2 * p.nx + 2 * side) {
-        x = p.nx - 1;
-        y = 1 + (k - 2 * p.nx - side);
-    } else {
-        return;
-    }
-    T f[9];
-    load_general<9, ST, ODD>(p, x, y, f);
-    diffusive_rule<T>(p, x, y, f);
-    store_general<9, ST, ODD>(p, x, y, f);
+    wall_site<ST, ODD>(p, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // Control-point probe: one thread appends the velocity of site probe_site
@@ -2555,7 +2584,6 @@ struct Launch {
     static cudaError_t fixup(int Q, int coll, bool odd, const Params& p, cudaStream_t s, int nsm);
     static cudaError_t prepass(int Q, int coll, bool odd, const Params& p, cudaStream_t s);
     static cudaError_t probe(int Q, bool odd, const Params& p, cudaStream_t s);
-    static cudaError_t walls(bool odd, const Params& p, cudaStream_t s);
     static cudaError_t init(int Q, const Params& p, const double* r, const double* ux,
                             const double* uy, int eqkind, cudaStream_t s);
     static cudaError_t init_uniform(int Q, const Params& p, double r, double ux, double uy,
@@ -2642,8 +2670,12 @@ cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
                             (uintptr_t)p.f % (2 * sizeof(typename ST::S)) == 0;
         if (paired) {
             dim3 b(kVecX, kVecY), g((p.nx + 2 * kVecX - 1) / (2 * kVecX), (p.ny + kVecY - 1) / kVecY);
-            return launch_p(odd ? step_kernel_v2<Q, ST, COLL, true> : step_kernel_v2<Q, ST, COLL, false>, g, b,
-                            s, p);
+            cudaError_t e = launch_p(odd ? step_kernel_v2<Q, ST, COLL, true> : step_kernel_v2<Q, ST, COLL, false>, g,
+                                     b, s, p);
+            if (e == cudaSuccess && p.diffusive)
+                e = launch_p(odd ? diffusive_wall_kernel<ST, true> : diffusive_wall_kernel<ST, false>,
+                             dim3((wall_sites(p) + 255) / 256), dim3(256), s, p);
+            return e;
         }
     }
     if constexpr (Q == 3 && COLL == LBM_ELBM && sizeof(typename ST::T) == 8)
@@ -2663,6 +2695,17 @@ cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
     if (kFlat<Q, ST>) {
         b = dim3(kFlatThreads);
         g = dim3((unsigned)(((int64_t)p.nx * p.ny + kFlatThreads - 1) / kFlatThreads));
+    }
+    if constexpr (Q == 9) {
+        if (p.diffusive) {
+            const int n = wall_sites(p);
+            if (kFlat<Q, ST>)
+                g.x += (n + kFlatThreads - 1) / kFlatThreads;
+            else
+                g.y += (n + (int)g.x * kBlockX * kBlockY - 1) / ((int)g.x * kBlockX * kBlockY);
+            return launch_p(odd ? step_kernel<Q, ST, COLL, true, true> : step_kernel<Q, ST, COLL, false, true>, g, b, s,
+                            p);
+        }
     }
     return launch_p(odd ? step_kernel<Q, ST, COLL, true> : step_kernel<Q, ST, COLL, false>, g, b, s, p);
 }
@@ -2755,13 +2798,6 @@ cudaError_t Launch<ST>::line(int coll, const Params& p, const void* src, int64_t
         case LBM_ELBM: return launch_line<ST, LBM_ELBM>(p, src, sp, dst, dp, threads, steps, halo, s);
     }
     return cudaErrorInvalidValue;
-}
-
-template <class ST>
-cudaError_t Launch<ST>::walls(bool odd, const Params& p, cudaStream_t s) {
-    const int n = 2 * p.nx + 2 * (p.ny - 2);
-    return launch_p(odd ? diffusive_wall_kernel<ST, true> : diffusive_wall_kernel<ST, false>,
-                    dim3((n + 255) / 256), dim3(256), s, p);
 }
 
 template <class ST>
