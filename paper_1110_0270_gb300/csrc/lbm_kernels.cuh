@@ -1347,11 +1347,19 @@ __device__ __forceinline__ double delta_s_lanes(const Params& p, double v, bool 
     double x = 0.0, fe = 0.0;
     bool neg = false;
     if (act) {
-        const double ri = 1.0 / r, ux = jx * ri, uy = jy * ri;
+        // (reciprocals and roots by Newton steps from an FP32 seed, the series by
+        // pairs: a chain of FP64 operations is 64 clocks each)
+        const double ri = rcp_f64(r), ux = jx * ri, uy = jy * ri;
         double ax[3], ay[3];
         if (p.eq == LBM_EQ_ENTROPIC) {
-            eq1d_entropic<double>(ux, ax[0], ax[1], ax[2]);
-            eq1d_entropic<double>(uy, ay[0], ay[1], ay[2]);
+            const double a = fma(sqrt_f64(fma(3.0 * ux, ux, 1.0)), 1.0 / 3.0, -1.0 / 6.0);
+            const double b = fma(sqrt_f64(fma(3.0 * uy, uy, 1.0)), 1.0 / 3.0, -1.0 / 6.0);
+            ax[0] = fma(-0.5, ux, a);
+            ax[1] = fma(-2.0, a, 1.0);
+            ax[2] = fma(0.5, ux, a);
+            ay[0] = fma(-0.5, uy, b);
+            ay[1] = fma(-2.0, b, 1.0);
+            ay[2] = fma(0.5, uy, b);
         } else {
             eq1d_poly<double>(ux, ax[0], ax[1], ax[2]);
             eq1d_poly<double>(uy, ay[0], ay[1], ay[2]);
@@ -1374,15 +1382,16 @@ __device__ __forceinline__ double delta_s_lanes(const Params& p, double v, bool 
         }
         const double d = inv != 0.0 ? (v - fe) * inv : v - fe;  // f - f*
         neg = (inv != 0.0 ? fe + d : v) < 0.0 || !(fe > 0.0);
-        x = d / fe;
+        x = d * rcp_f64(fe);
     }
     // one tier of gfun_d for the warp: the series (or log) its largest |x| needs
     const float axf = fminf((float)fabs(x), 2.0f);
     const float am = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(axf)));
-    double g;
-    if (am < 0.015625f) g = gseries_d<8>(x);
-    else if (am < 0.125f) g = gseries_d<16>(x);
-    else if (am < 0.25f) g = gseries_d<26>(x);
+    double g, ln;
+    if (am < 0.015625f) gl_pairs<8, 9>(x, g, ln);
+    else if (am < 0.125f) gl_artanh<7>(x, g, ln);
+    else if (am < 0.25f) gl_artanh<9>(x, g, ln);
+    else if (am < 0.5f) gl_artanh<17>(x, g, ln);
     else g = x <= -1.0 ? 1.0 : (1.0 + x) * log1p(x) - x;
     double term = act ? fe * g : 0.0;
 #pragma unroll
@@ -1634,6 +1643,49 @@ __device__ void threshold_select_apply(const Params& p, unsigned M) {
     }
 }
 
+// The post-collision state of a selected site with pre-collision populations f
+// written back: f*, or A_2 for the MRT limiter.  In FP64 on D2Q9 by the pair
+// sums of lbm_fp64.cuh: one thread's chain of FP64 operations (64 clocks each),
+// which the step waits for, is a third as long.
+template <int Q, class ST, int COLL, bool ODD>
+__device__ __forceinline__ void rewrite_selected(const Params& p, int site, const typename ST::T* f) {
+    using T = typename ST::T;
+    T feq[Q];
+    if constexpr (Q == 9 && sizeof(T) == 8) {
+        Eq64 m;
+        moments_f64(f, m);
+        if (p.eq != LBM_EQ_POLY_STD) factors_f64(p.eq, m);
+        T e[9];
+        if constexpr (COLL == LBM_MRT_LIMITER) {
+            diff_f64<0>(p.eq, m, f, e);
+            mrt2_f64(p.mrt2_c, f, e, feq);
+        } else if (p.eq == LBM_EQ_POLY_STD) {
+            diff_f64<0>(p.eq, m, f, e);
+#pragma unroll
+            for (int i = 1; i < 9; ++i) feq[i] = f[i] + e[i];
+        } else {
+#pragma unroll
+            for (int i = 1; i < 9; ++i) feq[i] = m.X[Lat<9>::cx(i) + 1] * m.Y[Lat<9>::cy(i) + 1];
+        }
+        mass_f64(m.rho, feq);
+        rewrite_site<Q, ST, ODD>(p, site, feq);
+    } else {
+        T rho, ux, uy;
+        moments<Q, T>(f, rho, ux, uy);
+        equilibrium<Q, T>(p.eq, rho, ux, uy, feq);
+        if constexpr (COLL == LBM_MRT_LIMITER && Q == 9) {
+            // Section 5's MRT limiter: the selected site takes A_2, not f*
+            T F[Q];
+            mrt2_d2q9<T>(f, feq, sizeof(T) == 8 ? T(2.0 * p.beta) : T(2) * T(p.beta_f), F);
+            conserve_mass<Q, T>(rho, F);
+            rewrite_site<Q, ST, ODD>(p, site, F);
+        } else {
+            conserve_mass<Q, T>(rho, feq);
+            rewrite_site<Q, ST, ODD>(p, site, feq);
+        }
+    }
+}
+
 // Runs in one CTA of any size after every cand_ds entry of the step is final
 // (the entries of other CTAs are read through L2).
 template <int Q, class ST, bool ODD, int COLL = LBM_EHRENFEST>
@@ -1756,20 +1808,9 @@ __device__ void ehrenfest_select_apply(const Params& p, unsigned M, unsigned nva
         }
         p.cand_sel[j] = sel ? 1 : 0;
         if (sel) {
-            T f[Q], feq[Q], rho, ux, uy;
+            T f[Q];
             load_candidate<Q, ST>(p, (int)j, f);
-            moments<Q, T>(f, rho, ux, uy);
-            equilibrium<Q, T>(p.eq, rho, ux, uy, feq);
-            if constexpr (COLL == LBM_MRT_LIMITER && Q == 9) {
-                // Section 5's MRT limiter: the selected site takes A_2, not f*
-                T F[Q];
-                mrt2_d2q9<T>(f, feq, sizeof(T) == 8 ? T(2.0 * p.beta) : T(2) * T(p.beta_f), F);
-                conserve_mass<Q, T>(rho, F);
-                rewrite_site<Q, ST, ODD>(p, (int)site, F);
-            } else {
-                conserve_mass<Q, T>(rho, feq);
-                rewrite_site<Q, ST, ODD>(p, (int)site, feq);
-            }
+            rewrite_selected<Q, ST, COLL, ODD>(p, (int)site, f);
             ++mine;
         }
     });
@@ -1792,58 +1833,57 @@ __device__ __forceinline__ void select_apply(const Params& p, unsigned M, unsign
         ehrenfest_select_apply<Q, ST, ODD, COLL>(p, M, nvalid);
 }
 
-// The post-collision state of selected record j written back (f*, or A_2
-// for the MRT limiter).
-template <int Q, class ST, int COLL, bool ODD>
-__device__ __forceinline__ void rewrite_selected(const Params& p, unsigned j) {
-    using T = typename ST::T;
-    T f[Q], feq[Q], rho, ux, uy;
-    load_candidate<Q, ST>(p, (int)j, f);
-    moments<Q, T>(f, rho, ux, uy);
-    equilibrium<Q, T>(p.eq, rho, ux, uy, feq);
-    const int site = p.cand_site[j];
-    if constexpr (COLL == LBM_MRT_LIMITER && Q == 9) {
-        T F[Q];
-        mrt2_d2q9<T>(f, feq, sizeof(T) == 8 ? T(2.0 * p.beta) : T(2) * T(p.beta_f), F);
-        conserve_mass<Q, T>(rho, F);
-        rewrite_site<Q, ST, ODD>(p, site, F);
-    } else {
-        conserve_mass<Q, T>(rho, feq);
-        rewrite_site<Q, ST, ODD>(p, site, feq);
-    }
-}
-
 constexpr int64_t kSettleSites = 1 << 21;
 
 // Up to two screened records per thread: every CTA settles every record's
 // side of delta in FP32 (certify_side; the same result in each CTA).  When
 // every side is settled and at most k records are above delta, the first
 // CTA takes all of those without FP64 work and the call returns true in
-// every CTA; otherwise it returns false everywhere and the grid-wide FP64
-// evaluation decides.  Out of line: inlined, its code in front of the other
-// paths slowed the selection kernel of large lattices (measured).
+// every CTA; otherwise it returns false everywhere and the FP64 evaluation
+// decides.  On a small lattice the step waits for this chain, so the record of
+// each thread is read beside the count, before it is known to be one (with
+// the count first, then the record, its site and, for a selected one, the
+// record again, 129^2 FP64 took 16.3 us a step, 13.2 this way).  M: the number of records, for the caller.  Out of
+// line: inlined, its code in front of the other paths slowed the selection
+// kernel of large lattices (measured).
 template <int Q, class ST, bool ODD, int COLL>
-__device__ __noinline__ bool settle_all_taken(const Params& p, unsigned M) {
+__device__ __noinline__ bool settle_all_taken(const Params& p, unsigned& M_) {
     using T = typename ST::T;
     const unsigned tid = threadIdx.x, nt = blockDim.x;
-    int side[2];
-    float ds32[2];
+    T f[Q];
+    int site = 0;
+    const unsigned* cnt = &p.counters[p.cslot];
+    if (tid < (unsigned)p.cand_cap) {
+        load_candidate<Q, ST>(p, (int)tid, f);
+        site = p.cand_site[tid];
+    } else {
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const unsigned j = tid + r * nt;
-        side[r] = 0;
-        ds32[r] = 0.f;
-        if (j < M) {
-            T f[Q];
-            float ff[Q];
-            load_candidate<Q, ST>(p, (int)j, f);
-#pragma unroll
-            for (int i = 0; i < Q; ++i) ff[i] = (float)f[i];
-            side[r] = certify_side<Q>(p, ff, ds32[r]);
-        }
+        for (int i = 0; i < Q; ++i) f[i] = T(1);
     }
+    unsigned M = *cnt;
+    if (M > (unsigned)p.cand_cap) M = (unsigned)p.cand_cap;
+    M_ = M;
+    if (M > 2 * nt) return false;
+    int side[2] = {0, 0};
+    float ds32[2] = {0.f, 0.f};
+    if (tid < M) {
+        float ff[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) ff[i] = (float)f[i];
+        side[0] = certify_side<Q>(p, ff, ds32[0]);
+    }
+    if (tid + nt < M) {
+        T f2[Q];
+        float ff[Q];
+        load_candidate<Q, ST>(p, (int)(tid + nt), f2);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) ff[i] = (float)f2[i];
+        side[1] = certify_side<Q>(p, ff, ds32[1]);
+    }
+    __syncwarp();
     const int unsure = __syncthreads_or(side[0] == 2 || side[1] == 2);
-    const unsigned nabove = (unsigned)__syncthreads_count(side[0] == 1) + (unsigned)__syncthreads_count(side[1] == 1);
+    unsigned nabove = (unsigned)__syncthreads_count(side[0] == 1);
+    if (M > nt) nabove += (unsigned)__syncthreads_count(side[1] == 1);
     const unsigned K = p.topk > 0 ? (unsigned)p.topk : 0u;
     if (unsure || nabove > K) return false;
     if (blockIdx.x != 0) return true;
@@ -1854,7 +1894,12 @@ __device__ __noinline__ bool settle_all_taken(const Params& p, unsigned M) {
         const bool sel = side[r] == 1;
         p.cand_sel[j] = sel ? 1 : 0;
         p.cand_ds[j] = sel ? (double)ds32[r] : -1.0;  // lbm_last_candidates recomputes FP64 values
-        if (sel) rewrite_selected<Q, ST, COLL, ODD>(p, j);
+        if (!sel) continue;
+        if (r == 1) {
+            load_candidate<Q, ST>(p, (int)j, f);
+            site = p.cand_site[j];
+        }
+        rewrite_selected<Q, ST, COLL, ODD>(p, site, f);
     }
     if (tid == 0) {
         p.counters[CNT_NVALID] = nabove;
@@ -1867,15 +1912,16 @@ __device__ __noinline__ bool settle_all_taken(const Params& p, unsigned M) {
 template <int Q, class ST, bool ODD, int COLL>
 __device__ __forceinline__ void eval_then_select(const Params& p) {
     __shared__ unsigned s_last;
-    unsigned M = p.counters[p.cslot];
-    if (M > (unsigned)p.cand_cap) M = (unsigned)p.cand_cap;
-    if constexpr (COLL != LBM_THRESHOLD) {
-        // small lattices only: there the selection's latency is most of the
-        // step, while on large ones the grid-wide pass hides under the next
-        // step's launch and a failed attempt would only add to it (measured)
-        if ((int64_t)p.nx * p.ny <= kSettleSites && M > (blockDim.x >> 4) && M <= 2 * blockDim.x &&
-            settle_all_taken<Q, ST, ODD, COLL>(p, M))
-            return;
+    unsigned M;
+    // small lattices only: there the selection's latency is most of the
+    // step, while on large ones the grid-wide pass hides under the next
+    // step's launch and a failed attempt would only add to it (measured)
+    const bool small = COLL != LBM_THRESHOLD && (int64_t)p.nx * p.ny <= kSettleSites;
+    if (small) {
+        if (settle_all_taken<Q, ST, ODD, COLL>(p, M)) return;
+    } else {
+        M = p.counters[p.cslot];
+        if (M > (unsigned)p.cand_cap) M = (unsigned)p.cand_cap;
     }
     if (M <= (blockDim.x >> 4)) {
         // few screened sites (the usual case): the first CTA evaluates them
@@ -1891,7 +1937,7 @@ __device__ __forceinline__ void eval_then_select(const Params& p) {
             s_last = 0;
             s_nsel = 0;
         }
-        if constexpr (COLL != LBM_THRESHOLD) {
+        if (COLL != LBM_THRESHOLD && !small) {
             // every screened site certainly on one side of delta in FP32 and
             // no more candidates than k: all of them are taken, no FP64
             // Delta S (FP64 storage: the records rounded to FP32 move Delta S
@@ -1917,21 +1963,7 @@ __device__ __forceinline__ void eval_then_select(const Params& p) {
                     // the FP32 value of a selected site (lbm_last_candidates
                     // recomputes FP64 values)
                     p.cand_ds[j] = sel ? (double)ds32 : -1.0;
-                    if (sel) {
-                        T feq[Q], rho, ux, uy;
-                        moments<Q, T>(f, rho, ux, uy);
-                        equilibrium<Q, T>(p.eq, rho, ux, uy, feq);
-                        const int site = p.cand_site[j];
-                        if constexpr (COLL == LBM_MRT_LIMITER && Q == 9) {
-                            T F[Q];
-                            mrt2_d2q9<T>(f, feq, sizeof(T) == 8 ? T(2.0 * p.beta) : T(2) * T(p.beta_f), F);
-                            conserve_mass<Q, T>(rho, F);
-                            rewrite_site<Q, ST, ODD>(p, site, F);
-                        } else {
-                            conserve_mass<Q, T>(rho, feq);
-                            rewrite_site<Q, ST, ODD>(p, site, feq);
-                        }
-                    }
+                    if (sel) rewrite_selected<Q, ST, COLL, ODD>(p, p.cand_site[j], f);
                 }
                 if (threadIdx.x == 0) {
                     p.counters[CNT_NVALID] = ncert;
@@ -1974,19 +2006,9 @@ __device__ __forceinline__ void eval_then_select(const Params& p) {
                 p.cand_sel[j] = sel ? 1 : 0;
                 if (sel) {
                     using T = typename ST::T;
-                    T f[Q], feq[Q], rho, ux, uy;
+                    T f[Q];
                     load_candidate<Q, ST>(p, (int)j, f);
-                    moments<Q, T>(f, rho, ux, uy);
-                    equilibrium<Q, T>(p.eq, rho, ux, uy, feq);
-                    if constexpr (COLL == LBM_MRT_LIMITER && Q == 9) {
-                        T F[Q];
-                        mrt2_d2q9<T>(f, feq, sizeof(T) == 8 ? T(2.0 * p.beta) : T(2) * T(p.beta_f), F);
-                        conserve_mass<Q, T>(rho, F);
-                        rewrite_site<Q, ST, ODD>(p, site, F);
-                    } else {
-                        conserve_mass<Q, T>(rho, feq);
-                        rewrite_site<Q, ST, ODD>(p, site, feq);
-                    }
+                    rewrite_selected<Q, ST, COLL, ODD>(p, site, f);
                     atomicAdd(&s_nsel, 1u);
                 }
             }
@@ -2240,17 +2262,29 @@ __global__ void __launch_bounds__(256) median_fixup(Params p) {
 template <int Q, class ST>
 __device__ __forceinline__ void median_homothety(const Params& p, int j, typename ST::T phi, typename ST::T* F) {
     using T = typename ST::T;
-    T f[Q], feq[Q], rho, ux, uy;
+    T f[Q];
     load_candidate<Q, ST>(p, j, f);
-    moments<Q, T>(f, rho, ux, uy);
-    equilibrium<Q, T>(p.eq, rho, ux, uy, feq);
-    const T om = T(2) * T(p.beta);
+    if constexpr (Q == 9 && sizeof(T) == 8) {
+        // F = f + (1 - (1 - 2 beta) phi) (f* - f) on the pair sums
+        Eq64 m;
+        double e[9];
+        moments_f64(f, m);
+        if (p.eq != LBM_EQ_POLY_STD) factors_f64(p.eq, m);
+        diff_f64<1>(p.eq, m, f, e);
+        lbgk_f64(fma(p.two_beta - 1.0, phi, 1.0), f, e, F);
+        mass_f64(m.rho, F);
+    } else {
+        T feq[Q], rho, ux, uy;
+        moments<Q, T>(f, rho, ux, uy);
+        equilibrium<Q, T>(p.eq, rho, ux, uy, feq);
+        const T om = T(2) * T(p.beta);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const T fl = feq[i] + phi * (f[i] - feq[i]);
-        F[i] = fl + om * (feq[i] - fl);
+        for (int i = 0; i < Q; ++i) {
+            const T fl = feq[i] + phi * (f[i] - feq[i]);
+            F[i] = fl + om * (feq[i] - fl);
+        }
+        conserve_mass<Q, T>(rho, F);
     }
-    conserve_mass<Q, T>(rho, F);
 }
 
 template <int Q>
@@ -2331,24 +2365,29 @@ __global__ void __launch_bounds__(256) median_recon_fixup(Params p) {
             bool sel = false;
             if (cand) {
                 ++nvalid;
-                double w[MW::W];
+                // the lower median by ranks, on the bits (the values are >= 0 or
+                // NaN, outside the window): integer compares, where an insertion
+                // sort was a chain of up to 36 FP64 ones
+                long long u[MW::W];
                 int n = 0;
 #pragma unroll
                 for (int kk = 0; kk < MW::W; ++kk) {
-                    const double u = win[kk];
-                    if (!(u == u)) continue;  // outside the window
-                    int m = n++;
-                    while (m > 0 && w[m - 1] > u) {  // insertion sort, ascending
-                        w[m] = w[m - 1];
-                        --m;
-                    }
-                    w[m] = u;
+                    u[kk] = __double_as_longlong(win[kk]) & 0x7fffffffffffffffLL;
+                    n += u[kk] <= 0x7ff0000000000000LL ? 1 : 0;
                 }
-                const double med = w[(n - 1) / 2];
+                long long mb = 0;
+#pragma unroll
+                for (int kk = 0; kk < MW::W; ++kk) {
+                    int rank = 0;
+#pragma unroll
+                    for (int l = 0; l < MW::W; ++l) rank += u[l] < u[kk] || (u[l] == u[kk] && l < kk) ? 1 : 0;
+                    if (rank == (n - 1) / 2) mb = u[kk];
+                }
+                const double med = __longlong_as_double(mb);
                 sel = med < c;
                 if (sel) {
                     ++nsel;
-                    const T phi = isinf(c) ? T(0) : T(sqrt(med / c));
+                    const T phi = isinf(c) ? T(0) : T(sqrt_f64(med * rcp_f64(c)));
                     if (direct) {
                         T F[Q];
                         median_homothety<Q, ST>(p, (int)j, phi, F);
