@@ -292,6 +292,21 @@ lbm_status reset_counters(lbm_ctx* ctx, cudaStream_t s) {
     return LBM_OK;
 }
 
+}  // namespace
+
+namespace lbm {
+lbm_status read_out(lbm_ctx* ctx, void* f, int dtype, bool after_kernel, cudaStream_t s) {
+    Params q = ctx->p;
+    q.pdl = after_kernel ? 1 : 0;
+    LBM_CK(ctx, dispatch(ctx->cfg.precision, [&](auto L) {
+               return decltype(L)::get_state(ctx->Q, q, f, dtype, ctx->parity != 0, s);
+           }));
+    return LBM_OK;
+}
+}  // namespace lbm
+
+namespace {
+
 // The lagged ensemble limiter's E(Delta S) for the first step of a new
 // state: the mean over that state itself (the unlagged limiter's pre-pass).
 lbm_status initial_mean(lbm_ctx* ctx, cudaStream_t s) {
@@ -307,8 +322,11 @@ lbm_status initial_mean(lbm_ctx* ctx, cudaStream_t s) {
 
 namespace {
 
-// The kernels of one step with counter slot `cslot` and A-A parity `odd`.
-cudaError_t enqueue_one_step(lbm_ctx* ctx, bool odd, int cslot, cudaStream_t s) {
+// The kernels of one step with counter slot `cslot` and A-A parity `odd`;
+// save: where the step keeps its pre-collision state (step_save), after_kernel
+// as for read_out.
+cudaError_t enqueue_one_step(lbm_ctx* ctx, bool odd, int cslot, cudaStream_t s, void* save = nullptr,
+                             bool after_kernel = true) {
     const int coll = ctx->cfg.collision;
     Params q = ctx->p;
     q.cslot = cslot;
@@ -321,8 +339,12 @@ cudaError_t enqueue_one_step(lbm_ctx* ctx, bool odd, int cslot, cudaStream_t s) 
         });
     if (e == cudaSuccess)
         e = traced(ctx, LBM_KERNEL_STEP, s, [&] {
-            return dispatch(ctx->cfg.precision,  // diffusive wall sites included
-                            [&](auto L) { return decltype(L)::step(ctx->Q, coll, odd, q, s); });
+            return dispatch(ctx->cfg.precision, [&](auto L) {  // diffusive wall sites included
+                if (!save) return decltype(L)::step(ctx->Q, coll, odd, q, s);
+                Params r = q;
+                if (!after_kernel) r.pdl = 0;
+                return decltype(L)::step_save(ctx->Q, coll, odd, r, save, s);
+            });
         });
     if (e == cudaSuccess && (limiter(coll) || coll == LBM_ENSEMBLE_LAGGED))
         e = traced(ctx, LBM_KERNEL_FIXUP, s, [&] {
@@ -333,6 +355,23 @@ cudaError_t enqueue_one_step(lbm_ctx* ctx, bool odd, int cslot, cudaStream_t s) 
         e = dispatch(ctx->cfg.precision, [&](auto L) { return decltype(L)::probe(ctx->Q, !odd, q, s); });
     return e;
 }
+
+}  // namespace
+
+namespace lbm {
+lbm_status step_saving(lbm_ctx* ctx, void* save, int dtype, bool after_kernel, cudaStream_t s) {
+    if (ctx->cfg.precision != LBM_FP64 && ctx->cfg.precision != LBM_FP32) {
+        const lbm_status st = read_out(ctx, save, dtype, after_kernel, s);
+        return st ? st : lbm_step(ctx, 1, s);
+    }
+    LBM_CK(ctx, enqueue_one_step(ctx, ctx->parity != 0, (int)(ctx->t & 1), s, save, after_kernel));
+    ctx->parity ^= 1;
+    ctx->t += 1;
+    return LBM_OK;
+}
+}  // namespace lbm
+
+namespace {
 
 // Captures `periods` A-A periods (even step with counter slot 0, odd with
 // slot 1, repeated) into *graph / *exec on a private stream.
@@ -598,10 +637,7 @@ lbm_status lbm_set_state(lbm_ctx* ctx, const void* f, int dtype, void* stream) {
 lbm_status lbm_get_state(lbm_ctx* ctx, void* f, int dtype, void* stream) {
     if (!ctx) return LBM_ERR_ARG;
     if (!f || (dtype != LBM_DTYPE_F64 && dtype != LBM_DTYPE_F32)) return fail(ctx, LBM_ERR_ARG, "bad state buffer or dtype");
-    LBM_CK(ctx, dispatch(ctx->cfg.precision, [&](auto L) {
-               return decltype(L)::get_state(ctx->Q, ctx->p, f, dtype, ctx->parity != 0, S(stream));
-           }));
-    return LBM_OK;
+    return lbm::read_out(ctx, f, dtype, false, S(stream));
 }
 
 lbm_status lbm_step(lbm_ctx* ctx, int nsteps, void* stream) {

@@ -90,6 +90,7 @@ AdjGeo geometry(const lbm_ctx* ctx) {
     g.periodic_y = ctx->p.periodic_y;
     g.eq = ctx->cfg.equilibrium;
     g.beta = ctx->p.beta;
+    g.beta_f = (float)ctx->p.beta;
     return g;
 }
 
@@ -136,8 +137,7 @@ lbm_status backward_t(lbm_ctx* ctx, int T_, int K, const void* seed, int seed_dt
         if (branches) ACK(ctx, cudaMemsetAsync(aux, 0xff, (size_t)len * N * sizeof(int), st));  // AUX_LBGK
         for (int k = 0; k < len; ++k) {
             const T* fk = (const T*)(w + L.seg + (size_t)k * L.dense);
-            AST(lbm_get_state(ctx, (void*)fk, dtype_of(ctx), st));
-            AST(lbm_step(ctx, 1, st));
+            AST(step_saving(ctx, (void*)fk, dtype_of(ctx), k > 0, st));
             if (branches)
                 ACK(ctx, AdjLaunch<T>::record(Q, ctx->p, coll, (int)((ctx->t - 1) & 1), fk, aux + (size_t)k * N,
                                               ctx->nsm, st));
@@ -146,7 +146,7 @@ lbm_status backward_t(lbm_ctx* ctx, int T_, int K, const void* seed, int seed_dt
         for (int k = len - 1; k >= 0; --k) {
             ACK(ctx, AdjLaunch<T>::step(Q, g, (const T*)(w + L.seg + (size_t)k * L.dense),
                                         branches ? aux + (size_t)k * N : nullptr, lam[c], lam[c ^ 1], acc, wbuf,
-                                        coll == LBM_MEDIAN, st));
+                                        coll == LBM_MEDIAN || coll == LBM_POSITIVITY, coll == LBM_MEDIAN, st));
             c ^= 1;
         }
         return LBM_OK;

@@ -34,6 +34,7 @@ struct AdjGeo {
     int nx, ny, periodic_x, periodic_y;
     int eq;  // equilibrium kind
     double beta;
+    float beta_f;
 };
 
 // 1D equilibrium (per unit density) and its derivative in u, both forms
@@ -116,6 +117,50 @@ __device__ __forceinline__ void block_add2(double v0, double v1, double* acc0, d
     }
 }
 
+// The adjoint step's two sums over the CTA: terms hi + lo in the arithmetic
+// type into *acc0, and u, nonzero on a few lid sites, into *acc1.  The 256
+// terms lie in shared memory and the first warp alone adds them in FP64; a
+// shuffle reduction of doubles in every warp spent more on the FP64 pipe (19
+// clocks of the SM per warp instruction, 24 of them a warp) than the step's
+// memory traffic takes (513^2 gradient, 400 steps: 22.6 -> 21.0 ms).  Every thread of a 256-thread CTA calls it once.
+template <class T>
+__device__ __forceinline__ void block_add_terms(T hi, T lo, double u, double* acc0, double* acc1) {
+    __shared__ T term[2][256];
+    __shared__ double lid[8];
+    __shared__ unsigned flag[8];
+    const unsigned full = 0xffffffffu;
+    const int t = threadIdx.x, w = t >> 5;
+    const bool some_lo = __any_sync(full, lo != T(0)), some_u = __any_sync(full, u != 0.0);
+    if (some_u)
+        for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(full, u, o);
+    if ((t & 31) == 0) {
+        lid[w] = u;
+        flag[w] = (some_lo ? 1u : 0u) | (some_u ? 2u : 0u);
+    }
+    term[0][t] = hi;
+    term[1][t] = lo;
+    __syncthreads();
+    if (t < 32) {
+        unsigned any = 0u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) any |= flag[k];
+        double a = 0.0;
+#pragma unroll
+        for (int k = 0; k < 256; k += 32) a += (double)term[0][k + t];
+        if (any & 1u)
+            for (int k = 0; k < 256; k += 32) a += (double)term[1][k + t];
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(full, a, o);
+        if (t == 0) {
+            if (a != 0.0) atomicAdd(acc0, a);
+            if (any & 2u) {
+                double b = 0.0;
+                for (int k = 0; k < 8; ++k) b += lid[k];
+                atomicAdd(acc1, b);
+            }
+        }
+    }
+}
+
 // Seed of J = 1/2 sum rho |u|^2: lambda_j = v_j . u - |u|^2 / 2, and J.
 template <int Q, class T>
 __global__ void __launch_bounds__(256) adj_seed_ke(AdjGeo g, const T* __restrict__ f, T* lam,
@@ -136,6 +181,9 @@ __global__ void __launch_bounds__(256) adj_seed_ke(AdjGeo g, const T* __restrict
     block_add2(e, 0.0, J, nullptr);
 }
 
+// The kernels of a segment are launched with programmatic dependence; what they
+// read was written by the kernels just before, so no pointer is __restrict__
+// (its loads could take the non-coherent path).
 // The adjoint kernels hold the rare FP64 branch work (median Delta S
 // gradients) in out-of-line functions and are compiled for four resident
 // CTAs per SM (two in FP64): the rare work spills instead of setting every site's
@@ -191,8 +239,9 @@ __device__ __forceinline__ void dense_site_d(const T* a, int64_t N, int64_t s, d
 // same precision, so the same decision).  The median's window site m: the
 // lower median of the clipped window's FP64 Delta S, ties by site index.
 template <int Q, class T>
-__global__ void __launch_bounds__(256, kAdjMinBlocks<T>) adj_record(Params p, int coll, int cslot, const T* __restrict__ f,
-                                                 int* __restrict__ aux) {
+__global__ void __launch_bounds__(256, kAdjMinBlocks<T>) adj_record(Params p, int coll, int cslot, const T* f,
+                                                 int* aux) {
+    pdl_enter();
     const int64_t N = (int64_t)p.nx * p.ny;
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
     if (coll == LBM_POSITIVITY) {
@@ -269,6 +318,40 @@ __global__ void __launch_bounds__(256, kAdjMinBlocks<T>) adj_record(Params p, in
     }
 }
 
+// Lambda_i at site (x, y): lambda_{t+1, i} of the neighbour along v_i, or
+// lambda_{t+1, opp(i)} of the site itself for a wall link; returns the lid
+// links' part of dJ/dU.  Addresses by selects, so that the loads go out
+// together (a branch per direction let each wait for the one before).
+template <int Q, class T>
+__device__ __forceinline__ double adj_gather(const AdjGeo& g, const T* lam_in, int N, int x, int y, int s,
+                                             T* Lam) {
+    using L = Lat<Q>;
+    // target columns and rows by v + 1
+    int xt[3] = {x - 1, x, x + 1}, yt[3] = {y - 1, y, y + 1};
+    if (g.periodic_x) {
+        xt[0] = x > 0 ? x - 1 : g.nx - 1;
+        xt[2] = x + 1 < g.nx ? x + 1 : 0;
+    }
+    if (g.periodic_y) {
+        yt[0] = y > 0 ? y - 1 : g.ny - 1;
+        yt[2] = y + 1 < g.ny ? y + 1 : 0;
+    }
+    const bool okx[3] = {xt[0] >= 0, true, xt[2] < g.nx}, oky[3] = {yt[0] >= 0, true, yt[2] < g.ny};
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const int a = L::cx(i) + 1, b = L::cy(i) + 1;
+        const bool in = okx[a] && oky[b];
+        Lam[i] = lam_in[in ? i * N + yt[b] * g.nx + xt[a] : L::opp(i) * N + s];  // Q N < 2^31
+    }
+    double dU = 0.0;
+    if (!oky[2]) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            if (L::cy(i) > 0) dU += (double)Lam[i] * (-6.0 * L::w(i) * L::cx(i));
+    }
+    return dU;
+}
+
 // The positivity and median branches of the adjoint step at site s (psi,
 // dpsi/dbeta, dpsi/df_j and the median's cross-term coefficient w), out of
 // line: they are rare, and the median's FP64 Delta S gradients would
@@ -280,7 +363,7 @@ struct AdjBranch {
 };
 
 template <int Q, class T>
-__device__ __noinline__ AdjBranch<Q, T> adj_branch(AdjGeo g, const T* __restrict__ f, int64_t N, int64_t s,
+__device__ __noinline__ AdjBranch<Q, T> adj_branch(AdjGeo g, const T* f, int64_t N, int64_t s,
                                                    int br, T gs) {
     using L = Lat<Q>;
     AdjBranch<Q, T> b;
@@ -338,31 +421,25 @@ __device__ __noinline__ AdjBranch<Q, T> adj_branch(AdjGeo g, const T* __restrict
 // dJ/dbeta in acc[1]; aux (NULL: every site LBGK) holds each site's branch.
 // For a median site the coefficient w = g (1 - 2 beta) sqrt(M / C) / (2 M) of
 // its cross term goes to wbuf[s] (adj_median_cross adds it at m).
-template <int Q, class T>
-__global__ void __launch_bounds__(256, kAdjMinBlocks<T>)
-    adj_step(AdjGeo g, const T* __restrict__ f, const int* __restrict__ aux, const T* __restrict__ lam_in,
-             T* __restrict__ lam_out, double* acc, double* __restrict__ wbuf) {
+// RARE: some sites may be of the median's or the positivity rule's branches
+// (LBGK and Ehrenfest steps have none, and without the call five CTAs per SM
+// instead of four).
+template <int Q, class T, bool RARE>
+__global__ void __launch_bounds__(256, RARE || sizeof(T) == 8 ? kAdjMinBlocks<T> : 5)
+    adj_step(AdjGeo g, const T* f, const int* aux, const T* lam_in,
+             T* lam_out, double* acc, double* wbuf) {
+    pdl_enter();
     using L = Lat<Q>;
-    const int64_t N = (int64_t)g.nx * g.ny;
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double dU = 0.0, dB = 0.0;
+    const int N = g.nx * g.ny, s = blockIdx.x * blockDim.x + threadIdx.x;  // Q N < 2^31: 32-bit offsets
+    double dU = 0.0;
+    T dB = T(0), dBlo = T(0);
     if (s < N) {
-        const int x = (int)s % g.nx, y = (int)s / g.nx;  // N < 2^31
+        const int y = s / g.nx, x = s - y * g.nx;
         T Lam[Q];
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            int tx = x + L::cx(i), ty = y + L::cy(i);
-            if (g.periodic_x) tx = tx < 0 ? tx + g.nx : (tx >= g.nx ? tx - g.nx : tx);
-            if (g.periodic_y) ty = ty < 0 ? ty + g.ny : (ty >= g.ny ? ty - g.ny : ty);
-            if (tx >= 0 && tx < g.nx && ty >= 0 && ty < g.ny) {
-                Lam[i] = lam_in[(int64_t)i * N + (int64_t)ty * g.nx + tx];
-            } else {
-                Lam[i] = lam_in[(int64_t)L::opp(i) * N + s];
-                if (ty >= g.ny) dU += (double)Lam[i] * (-6.0 * L::w(i) * L::cx(i));
-            }
-        }
+        dU = adj_gather<Q, T>(g, lam_in, N, x, y, s, Lam);
         T fs[Q], feq[Q], dr[Q], dx[Q], dy[Q], rho, ux, uy;
-        dense_site<Q, T>(f, N, s, fs);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) fs[i] = f[i * N + s];
         moments<Q, T>(fs, rho, ux, uy);
         eq_partials<Q, T>(g.eq, rho, ux, uy, feq, dr, dx, dy);
         T A = T(0), Bx = T(0), By = T(0), gs = T(0);
@@ -375,34 +452,47 @@ __global__ void __launch_bounds__(256, kAdjMinBlocks<T>)
         }
         const T inv = T(1) / rho;
         const int br = aux ? aux[s] : AUX_LBGK;
-        T psi = T(1) - T(2) * T(g.beta), dpsi_db = T(-2), dpsi[Q];
+        T psi = T(1) - T(2) * (sizeof(T) == 8 ? T(g.beta) : T(g.beta_f)), dpsi_db = T(-2), dpsi[Q];
+        T zero = T(0);
+        if constexpr (!RARE) {
+            // opaque, so that both instantiations round alike
+            if constexpr (sizeof(T) == 4)
+                asm("" : "+f"(zero));
+            else
+                asm("" : "+d"(zero));
+        }
 #pragma unroll
-        for (int j = 0; j < Q; ++j) dpsi[j] = T(0);
+        for (int j = 0; j < Q; ++j) dpsi[j] = zero;
         if (br == AUX_FSTAR) {
             psi = T(0);
             dpsi_db = T(0);
-        } else if (br != AUX_LBGK) {
-            const AdjBranch<Q, T> b = adj_branch<Q, T>(g, f, N, s, br, gs);
-            psi = b.psi;
-            dpsi_db = b.dpsi_db;
+        }
+        if constexpr (RARE) {
+            if (br != AUX_FSTAR && br != AUX_LBGK) {
+                const AdjBranch<Q, T> b = adj_branch<Q, T>(g, f, N, s, br, gs);
+                psi = b.psi;
+                dpsi_db = b.dpsi_db;
 #pragma unroll
-            for (int j = 0; j < Q; ++j) dpsi[j] = b.dpsi[j];
-            if (br >= 0) wbuf[s] = b.w;
+                for (int j = 0; j < Q; ++j) dpsi[j] = b.dpsi[j];
+                if (br >= 0) wbuf[s] = b.w;
+            }
         }
 #pragma unroll
         for (int j = 0; j < Q; ++j) {
             const T a = A + Bx * (T(L::cx(j)) - ux) * inv + By * (T(L::cy(j)) - uy) * inv;
-            lam_out[(int64_t)j * N + s] = (T(1) - psi) * a + psi * Lam[j] + gs * dpsi[j];
+            lam_out[j * N + s] = (T(1) - psi) * a + psi * Lam[j] + gs * dpsi[j];
         }
-        dB = (double)gs * (double)dpsi_db;
+        dB = gs * dpsi_db;
+        // the product's rounding (none for -2 and 0)
+        if (sizeof(T) == 4 && fabs(dB) < T(INFINITY)) dBlo = fma(gs, dpsi_db, -dB);
     }
-    block_add2(dU, dB, acc, acc + 1);
+    block_add_terms<T>(dB, dBlo, dU, acc + 1, acc);
 }
 
 // The median's cross term: a selected site s with window site m = aux[s]
 // adds wbuf[s] dM/df(m) to lambda_t(m) (after adj_step has written it).
 template <int Q, class T>
-__device__ __noinline__ void adj_cross_site(AdjGeo g, const T* __restrict__ f, int64_t N, int m, double w,
+__device__ __noinline__ void adj_cross_site(AdjGeo g, const T* f, int64_t N, int m, double w,
                                             T* lam_out) {
     double fm[Q], gM[Q];
     dense_site_d<Q, T>(f, N, m, fm);
@@ -412,9 +502,10 @@ __device__ __noinline__ void adj_cross_site(AdjGeo g, const T* __restrict__ f, i
 }
 
 template <int Q, class T>
-__global__ void __launch_bounds__(256, kAdjMinBlocks<T>) adj_median_cross(AdjGeo g, const T* __restrict__ f,
-                                                       const int* __restrict__ aux,
-                                                       const double* __restrict__ wbuf, T* lam_out) {
+__global__ void __launch_bounds__(256, kAdjMinBlocks<T>) adj_median_cross(AdjGeo g, const T* f,
+                                                       const int* aux,
+                                                       const double* wbuf, T* lam_out) {
+    pdl_enter();
     const int N = g.nx * g.ny;  // < 2^31
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < N; s += gridDim.x * blockDim.x) {
         const int m = aux[s];
@@ -443,31 +534,23 @@ struct AdjLaunch {
         return cudaGetLastError();
     }
     static cudaError_t step(int Q, const AdjGeo& g, const T* f, const int* aux, const T* lin, T* lout,
-                            double* acc, double* wbuf, bool median, cudaStream_t s) {
+                            double* acc, double* wbuf, bool rare, bool median, cudaStream_t s) {
         const int64_t N = (int64_t)g.nx * g.ny;
         const unsigned blocks = (unsigned)((N + 255) / 256);
-        if (Q == 3)
-            adj_step<3, T><<<blocks, 256, 0, s>>>(g, f, aux, lin, lout, acc, wbuf);
-        else
-            adj_step<9, T><<<blocks, 256, 0, s>>>(g, f, aux, lin, lout, acc, wbuf);
-        cudaError_t e = cudaGetLastError();
+        void (*k)(AdjGeo, const T*, const int*, const T*, T*, double*, double*) =
+            rare ? (Q == 3 ? adj_step<3, T, true> : adj_step<9, T, true>)
+                 : (Q == 3 ? adj_step<3, T, false> : adj_step<9, T, false>);
+        cudaError_t e = launch_pdl(k, blocks, 256, s, g, f, aux, lin, lout, acc, wbuf);
         if (e != cudaSuccess || !median) return e;
-        if (Q == 3)
-            adj_median_cross<3, T><<<blocks, 256, 0, s>>>(g, f, aux, wbuf, lout);
-        else
-            adj_median_cross<9, T><<<blocks, 256, 0, s>>>(g, f, aux, wbuf, lout);
-        return cudaGetLastError();
+        return launch_pdl(Q == 3 ? adj_median_cross<3, T> : adj_median_cross<9, T>, blocks, 256, s, g, f, aux,
+                          (const double*)wbuf, lout);
     }
     static cudaError_t record(int Q, const Params& p, int coll, int cslot, const T* f, int* aux, int nsm,
                               cudaStream_t s) {
         const int64_t N = (int64_t)p.nx * p.ny;
         const unsigned blocks =
             coll == LBM_POSITIVITY ? (unsigned)std::min<int64_t>((N + 255) / 256, 8 * nsm) : (unsigned)nsm;
-        if (Q == 3)
-            adj_record<3, T><<<blocks, 256, 0, s>>>(p, coll, cslot, f, aux);
-        else
-            adj_record<9, T><<<blocks, 256, 0, s>>>(p, coll, cslot, f, aux);
-        return cudaGetLastError();
+        return launch_pdl(Q == 3 ? adj_record<3, T> : adj_record<9, T>, blocks, 256, s, p, coll, cslot, f, aux);
     }
     template <class U>
     static cudaError_t convert(const T* a, U* b, int64_t n, cudaStream_t s) {

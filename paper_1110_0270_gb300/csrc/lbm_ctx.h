@@ -47,3 +47,10 @@ struct lbm_ctx {
     }
 };
 
+namespace lbm {
+// lbm_get_state's transfer; after_kernel: the stream's last operation is a
+// kernel, on which the launch may depend programmatically.
+lbm_status read_out(lbm_ctx* ctx, void* f, int dtype, bool after_kernel, cudaStream_t s);
+// One step that leaves its pre-collision state in save (as read_out would).
+lbm_status step_saving(lbm_ctx* ctx, void* save, int dtype, bool after_kernel, cudaStream_t s);
+}  // namespace lbm

@@ -824,9 +824,11 @@ constexpr bool kLimForm = Q == 9 && sizeof(typename ST::T) == 4 &&
                           (COLL == LBM_SMOOTH || COLL == LBM_DOUBLE_MONOTONIC || COLL == LBM_ENSEMBLE ||
                            COLL == LBM_THRESHOLD || COLL == LBM_ENSEMBLE_LAGGED);
 
+// save (FP64 and FP32 storage): the pre-collision populations also go there,
+// dense [Q][ny][nx].
 template <int Q, class ST, int COLL, bool ODD>
 __device__ __forceinline__ void site_update(const Params& p, int x, int y, int& e_code,
-                                            int& e_iters, typename ST::T& acc) {
+                                            int& e_iters, typename ST::T& acc, typename ST::T* save = nullptr) {
     using T = typename ST::T;
     constexpr bool DEV = kDeviationForm<Q, ST, COLL>;
     T f[Q], F[Q];
@@ -842,6 +844,11 @@ __device__ __forceinline__ void site_update(const Params& p, int x, int y, int& 
         load_interior<Q, ST, ODD, DEV>(p, o, f);
     else
         load_general<Q, ST, ODD, DEV>(p, x, y, f);
+    if (save) {
+        const int64_t N = (int64_t)p.nx * p.ny;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) save[i * N + (y * p.nx + x)] = f[i];
+    }
     if constexpr (DEV) {
         collide_dev<float, ST, COLL>(p, x, y, f, F);
     } else if constexpr (kLimForm<Q, ST, COLL>) {
@@ -1017,9 +1024,8 @@ constexpr int kFlatThreads = 64;
 // WALLS (diffusive walls): the CTAs behind the lattice's own take the wall
 // sites, beside the collisions instead of in a kernel after them (6 us
 // of a 28 us step of the 100^2 box in FP64).
-template <int Q, class ST, int COLL, bool ODD, bool WALLS = false>
-__global__ void __launch_bounds__(kBlockX* kBlockY, kMinBlocks<ST, COLL>) step_kernel(Params p) {
-    pdl_enter();
+template <int Q, class ST, int COLL, bool ODD, bool WALLS>
+__device__ __forceinline__ void step_body(const Params& p, typename ST::T* save) {
     int x, y;
     if constexpr (kFlat<Q, ST>) {
         const unsigned s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1056,11 +1062,32 @@ __global__ void __launch_bounds__(kBlockX* kBlockY, kMinBlocks<ST, COLL>) step_k
     if constexpr (kElbmWarp<ST, COLL>)
         elbm_update<Q, ST, ODD>(p, x, y, x < p.nx && y < p.ny, e_code, e_iters);
     else if (x < p.nx && y < p.ny)
-        site_update<Q, ST, COLL, ODD>(p, x, y, e_code, e_iters, acc);
+        site_update<Q, ST, COLL, ODD>(p, x, y, e_code, e_iters, acc, save);
     if (COLL == LBM_ELBM) elbm_stats(p, e_code, e_iters);
     if (COLL == LBM_THRESHOLD) block_sum_to_slots<typename ST::T>(p, acc, 0, false);
     if (COLL == LBM_ENSEMBLE_LAGGED)
         block_sum_to_slots<typename ST::T>(p, acc, e_code == 1 ? typename ST::T(1) : typename ST::T(0), true);
+}
+
+template <int Q, class ST, int COLL, bool ODD, bool WALLS = false>
+__global__ void __launch_bounds__(kBlockX* kBlockY, kMinBlocks<ST, COLL>) step_kernel(Params p) {
+    pdl_enter();
+    step_body<Q, ST, COLL, ODD, WALLS>(p, nullptr);
+}
+
+// The same, keeping the pre-collision state (the adjoint's recomputation): the
+// populations are in registers anyway, where a kernel of its own that copied
+// them read the lattice once more and took a launch (513^2 gradient, 400
+// steps, with the segment's kernels launched ahead: 17.8 -> 15.8 ms).
+template <class ST, int COLL>
+constexpr bool kSaveForm = sizeof(typename ST::S) == sizeof(typename ST::T) &&
+                           (COLL == LBM_LBGK || COLL == LBM_EHRENFEST || COLL == LBM_MEDIAN || COLL == LBM_POSITIVITY);
+
+template <int Q, class ST, int COLL, bool ODD>
+__global__ void __launch_bounds__(kBlockX* kBlockY, kMinBlocks<ST, COLL>)
+    step_save_kernel(Params p, typename ST::T* save) {
+    pdl_enter();
+    step_body<Q, ST, COLL, ODD, false>(p, save);
 }
 
 // Several steps of a D1Q3 line in one launch, for the collisions that need
@@ -2510,6 +2537,7 @@ __device__ __forceinline__ void read_state(const Params& p, int x, int y, bool o
 
 template <int Q, class ST, class Out>
 __global__ void get_state_kernel(Params p, Out* dst, int odd) {
+    pdl_enter();
     using T = typename ST::T;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -2629,6 +2657,9 @@ __global__ void __launch_bounds__(256) entropy_kernel(Params p, double* H, doubl
 template <class ST>
 struct Launch {
     static cudaError_t step(int Q, int coll, bool odd, const Params& p, cudaStream_t s);
+    // step that keeps the pre-collision state in save; cudaErrorNotSupported
+    // for the forms without (16-bit storage, other collisions)
+    static cudaError_t step_save(int Q, int coll, bool odd, const Params& p, void* save, cudaStream_t s);
     static cudaError_t line(int coll, const Params& p, const void* src, int64_t sp, void* dst, int64_t dp, int threads,
                             int steps, int halo, cudaStream_t s);
     static cudaError_t fixup(int Q, int coll, bool odd, const Params& p, cudaStream_t s, int nsm);
@@ -2711,6 +2742,25 @@ inline dim3 site_block(int Q) { return Q == 3 ? dim3(256, 1) : dim3(kBlockX, kBl
 // against 49; 20000 sites, where the warps fill the FP64 pipes: 58 us against 55).
 constexpr int kElbmLaneMost = 16000;
 
+// CTA and grid of the one-site step kernel.
+template <int Q, class ST>
+void step_shape(const Params& p, dim3& b, dim3& g) {
+    b = site_block(Q);
+    if (Q == 3) {
+        // a D1Q3 line has few sites (the 800-site tube): spread them over the
+        // SMs in CTAs of as few as 32 threads, so that the ELBM root finder's
+        // FP64 chains and the limiter steps run on many SMs at once
+        const int nsm = p.pipe_ctas >= 8 ? p.pipe_ctas / 8 : 1;
+        int t = ((p.nx + nsm - 1) / nsm + 31) / 32 * 32;
+        b = dim3(t < 32 ? 32 : (t > 256 ? 256 : t), 1);
+    }
+    g = site_grid(p, b);
+    if (kFlat<Q, ST>) {
+        b = dim3(kFlatThreads);
+        g = dim3((unsigned)(((int64_t)p.nx * p.ny + kFlatThreads - 1) / kFlatThreads));
+    }
+}
+
 template <int Q, class ST, int COLL>
 cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
     // two sites per thread where every row starts on a pair boundary (the
@@ -2732,20 +2782,8 @@ cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
         if (p.nx <= kElbmLaneMost)
             return launch_p(odd ? elbm_lanes_step<ST, true> : elbm_lanes_step<ST, false>,
                             dim3((p.nx + kLaneSites - 1) / kLaneSites), dim3(32), s, p);
-    dim3 b = site_block(Q);
-    if (Q == 3) {
-        // a D1Q3 line has few sites (the 800-site tube): spread them over the
-        // SMs in CTAs of as few as 32 threads, so that the ELBM root finder's
-        // FP64 chains and the limiter steps run on many SMs at once
-        const int nsm = p.pipe_ctas >= 8 ? p.pipe_ctas / 8 : 1;
-        int t = ((p.nx + nsm - 1) / nsm + 31) / 32 * 32;
-        b = dim3(t < 32 ? 32 : (t > 256 ? 256 : t), 1);
-    }
-    dim3 g = site_grid(p, b);
-    if (kFlat<Q, ST>) {
-        b = dim3(kFlatThreads);
-        g = dim3((unsigned)(((int64_t)p.nx * p.ny + kFlatThreads - 1) / kFlatThreads));
-    }
+    dim3 b, g;
+    step_shape<Q, ST>(p, b, g);
     if constexpr (Q == 9) {
         if (p.diffusive) {
             const int n = wall_sites(p);
@@ -2824,6 +2862,37 @@ cudaError_t launch_prepass_q(int coll, bool odd, const Params& p, cudaStream_t s
 template <class ST>
 cudaError_t Launch<ST>::step(int Q, int coll, bool odd, const Params& p, cudaStream_t s) {
     return Q == 3 ? launch_step_c<3, ST>(coll, odd, p, s) : launch_step_c<9, ST>(coll, odd, p, s);
+}
+
+template <int Q, class ST, int COLL>
+cudaError_t launch_save_q(bool odd, const Params& p, void* save, cudaStream_t s) {
+    if constexpr (kSaveForm<ST, COLL>) {
+        dim3 b, g;
+        step_shape<Q, ST>(p, b, g);
+        void (*k)(Params, typename ST::T*) = odd ? step_save_kernel<Q, ST, COLL, true> : step_save_kernel<Q, ST, COLL, false>;
+        if (p.pdl) return launch_pdl(k, g, b, s, p, (typename ST::T*)save);
+        k<<<g, b, 0, s>>>(p, (typename ST::T*)save);
+        return cudaGetLastError();
+    }
+    return cudaErrorNotSupported;
+}
+
+template <int Q, class ST>
+cudaError_t launch_save_c(int coll, bool odd, const Params& p, void* save, cudaStream_t s) {
+    switch (coll) {
+        case LBM_LBGK: return launch_save_q<Q, ST, LBM_LBGK>(odd, p, save, s);
+        case LBM_EHRENFEST: return launch_save_q<Q, ST, LBM_EHRENFEST>(odd, p, save, s);
+        case LBM_POSITIVITY: return launch_save_q<Q, ST, LBM_POSITIVITY>(odd, p, save, s);
+        case LBM_MEDIAN:  // as launch_step_c
+            return p.median_inv != 0.0 ? launch_save_q<Q, ST, LBM_EHRENFEST>(odd, p, save, s)
+                                       : launch_save_q<Q, ST, LBM_MEDIAN>(odd, p, save, s);
+    }
+    return cudaErrorNotSupported;
+}
+
+template <class ST>
+cudaError_t Launch<ST>::step_save(int Q, int coll, bool odd, const Params& p, void* save, cudaStream_t s) {
+    return Q == 3 ? launch_save_c<3, ST>(coll, odd, p, save, s) : launch_save_c<9, ST>(coll, odd, p, save, s);
 }
 
 template <class ST, int COLL>
@@ -2917,22 +2986,20 @@ cudaError_t Launch<ST>::set_state(int Q, const Params& p, const void* src, int d
     return cudaGetLastError();
 }
 
+template <class ST, class Out>
+cudaError_t launch_get_state(int Q, const Params& p, Out* dst, bool odd, cudaStream_t s) {
+    const dim3 b = site_block(Q), g = site_grid(p, b);
+    void (*k)(Params, Out*, int) = Q == 3 ? get_state_kernel<3, ST, Out> : get_state_kernel<9, ST, Out>;
+    if (p.pdl) return launch_pdl(k, g, b, s, p, dst, odd ? 1 : 0);
+    k<<<g, b, 0, s>>>(p, dst, odd ? 1 : 0);
+    return cudaGetLastError();
+}
+
 template <class ST>
 cudaError_t Launch<ST>::get_state(int Q, const Params& p, void* dst, int dtype, bool odd,
                                   cudaStream_t s) {
-    dim3 b = site_block(Q), g = site_grid(p, b);
-    if (dtype == LBM_DTYPE_F64) {
-        if (Q == 3)
-            get_state_kernel<3, ST, double><<<g, b, 0, s>>>(p, (double*)dst, odd);
-        else
-            get_state_kernel<9, ST, double><<<g, b, 0, s>>>(p, (double*)dst, odd);
-    } else {
-        if (Q == 3)
-            get_state_kernel<3, ST, float><<<g, b, 0, s>>>(p, (float*)dst, odd);
-        else
-            get_state_kernel<9, ST, float><<<g, b, 0, s>>>(p, (float*)dst, odd);
-    }
-    return cudaGetLastError();
+    return dtype == LBM_DTYPE_F64 ? launch_get_state<ST, double>(Q, p, (double*)dst, odd, s)
+                                  : launch_get_state<ST, float>(Q, p, (float*)dst, odd, s);
 }
 
 template <class ST>
