@@ -2295,13 +2295,12 @@ __global__ void __launch_bounds__(256) median_fixup(Params p) {
 // recovered from the lattice, and the rewrites wait for every window of
 // the step: each selected site's coefficient goes to its record and the
 // last CTA to finish (ticket after a fence) writes the new populations.
-// The post-collision state of median candidate j whose pre-collision state
+// The post-collision state of a median candidate whose pre-collision state f
 // gets the homothety with coefficient phi before the LBGK collision.
 template <int Q, class ST>
-__device__ __forceinline__ void median_homothety(const Params& p, int j, typename ST::T phi, typename ST::T* F) {
+__device__ __forceinline__ void median_homothety(const Params& p, const typename ST::T* f, typename ST::T phi,
+                                                 typename ST::T* F) {
     using T = typename ST::T;
-    T f[Q];
-    load_candidate<Q, ST>(p, j, f);
     if constexpr (Q == 9 && sizeof(T) == 8) {
         // F = f + (1 - (1 - 2 beta) phi) (f* - f) on the pair sums
         Eq64 m;
@@ -2340,6 +2339,16 @@ __global__ void __launch_bounds__(256) median_recon_fixup(Params p) {
     using MW = MedWin<Q>;
     __shared__ double win[MW::W];
     __shared__ unsigned s_last;
+    // this CTA's first record is read beside the count, its populations (for
+    // the rewrite) by the thread that writes
+    constexpr unsigned kWriter = 16 * MW::centre;
+    int site = 0;
+    T fr[Q];
+    auto fetch = [&](unsigned j) {
+        site = p.cand_site[j];
+        if (threadIdx.x == kWriter) load_candidate<Q, ST>(p, (int)j, fr);
+    };
+    if (blockIdx.x < (unsigned)p.cand_cap) fetch(blockIdx.x);
     unsigned M = p.counters[p.cslot];
     if (M > (unsigned)p.cand_cap) M = (unsigned)p.cand_cap;
     const bool direct = M <= kMedDirect;
@@ -2356,13 +2365,13 @@ __global__ void __launch_bounds__(256) median_recon_fixup(Params p) {
     T* cf = (T*)p.cand_f;
     unsigned nvalid = 0, nsel = 0;
     for (unsigned j = blockIdx.x; j < M; j += gridDim.x) {
+        if (j != blockIdx.x) fetch(j);
         if (warp_works) {
             const bool act = k < (unsigned)MW::W;
             const bool centre = k == (unsigned)MW::centre;
             int xx = 0, yy = 0;
             bool inw = false;
             if (act) {
-                const int site = p.cand_site[j];
                 xx = site % p.nx + dx;
                 yy = site / p.nx + dy;
                 if (p.periodic_x) xx = xx < 0 ? xx + p.nx : (xx >= p.nx ? xx - p.nx : xx);
@@ -2396,50 +2405,44 @@ __global__ void __launch_bounds__(256) median_recon_fixup(Params p) {
             if (q == 0 && act) win[k] = inw ? ds : __longlong_as_double(0x7ff8000000000000LL);
         }
         __syncthreads();
-        if (threadIdx.x == 16 * MW::centre) {
-            const double c = win[MW::centre];
-            const bool cand = c > p.delta;
-            p.cand_ds[j] = cand ? c : -1.0;
-            bool sel = false;
-            if (cand) {
-                ++nvalid;
-                // the lower median by ranks, on the bits (the values are >= 0 or
-                // NaN, outside the window): integer compares, where an insertion
-                // sort was a chain of up to 36 FP64 ones
-                long long u[MW::W];
-                int n = 0;
+        if (threadIdx.x / 32 == kWriter / 32) {
+            // the lower median by ranks on the bits, a window site per lane (the
+            // values are >= 0, or NaN outside the window): one thread's insertion
+            // sort was a chain of up to 36 FP64 compares
+            const int l = threadIdx.x & 31;
+            const double v = l < MW::W ? win[l] : __longlong_as_double(0x7ff8000000000000LL);
+            const long long u = __double_as_longlong(v) & 0x7fffffffffffffffLL;
+            const int n = __popc(__ballot_sync(0xffffffffu, u <= 0x7ff0000000000000LL));
+            int rank = 0;
 #pragma unroll
-                for (int kk = 0; kk < MW::W; ++kk) {
-                    u[kk] = __double_as_longlong(win[kk]) & 0x7fffffffffffffffLL;
-                    n += u[kk] <= 0x7ff0000000000000LL ? 1 : 0;
-                }
-                long long mb = 0;
-#pragma unroll
-                for (int kk = 0; kk < MW::W; ++kk) {
-                    int rank = 0;
-#pragma unroll
-                    for (int l = 0; l < MW::W; ++l) rank += u[l] < u[kk] || (u[l] == u[kk] && l < kk) ? 1 : 0;
-                    if (rank == (n - 1) / 2) mb = u[kk];
-                }
-                const double med = __longlong_as_double(mb);
-                sel = med < c;
+            for (int k2 = 0; k2 < MW::W; ++k2) {
+                const long long o = __shfl_sync(0xffffffffu, u, k2);
+                rank += o < u || (o == u && k2 < l) ? 1 : 0;
+            }
+            const unsigned hit = __ballot_sync(0xffffffffu, l < MW::W && rank == (n - 1) / 2);
+            const double med = __longlong_as_double(__shfl_sync(0xffffffffu, u, hit ? __ffs(hit) - 1 : 0));
+            if (threadIdx.x == kWriter) {
+                const double c = win[MW::centre];
+                const bool cand = c > p.delta, sel = cand && med < c;
+                p.cand_ds[j] = cand ? c : -1.0;
+                p.cand_sel[j] = sel ? 1 : 0;
+                nvalid += cand ? 1 : 0;
+                nsel += sel ? 1 : 0;
                 if (sel) {
-                    ++nsel;
                     const T phi = isinf(c) ? T(0) : T(sqrt_f64(med * rcp_f64(c)));
                     if (direct) {
                         T F[Q];
-                        median_homothety<Q, ST>(p, (int)j, phi, F);
-                        rewrite_site<Q, ST, ODD>(p, p.cand_site[j], F);
+                        median_homothety<Q, ST>(p, fr, phi, F);
+                        rewrite_site<Q, ST, ODD>(p, site, F);
                     } else {
                         p.cand_ds[j] = (double)phi;  // for the last CTA (lbm_last_candidates recomputes Delta S)
                     }
                 }
             }
-            p.cand_sel[j] = sel ? 1 : 0;
         }
         __syncthreads();  // win is reused
     }
-    if (threadIdx.x == 16 * MW::centre) {
+    if (threadIdx.x == kWriter) {
         if (nvalid) atomicAdd(&p.counters[CNT_NVALID], nvalid);
         if (nsel) atomicAdd(&p.stats[ST_LIMITED], (unsigned long long)nsel);
     }
@@ -2452,8 +2455,9 @@ __global__ void __launch_bounds__(256) median_recon_fixup(Params p) {
     __threadfence();
     for (unsigned j = threadIdx.x; j < M; j += blockDim.x) {
         if (!__ldcg(&p.cand_sel[j])) continue;
-        T F[Q];
-        median_homothety<Q, ST>(p, (int)j, (T)__ldcg(&p.cand_ds[j]), F);
+        T f[Q], F[Q];
+        load_candidate<Q, ST>(p, (int)j, f);
+        median_homothety<Q, ST>(p, f, (T)__ldcg(&p.cand_ds[j]), F);
         rewrite_site<Q, ST, ODD>(p, p.cand_site[j], F);
     }
     if (threadIdx.x == 0) p.counters[CNT_DONE] = 0u;
@@ -2566,9 +2570,16 @@ __global__ void probe_kernel(Params p, int odd) {
     using T = typename ST::T;
     T f[Q], rho, ux, uy;
     const int x = p.probe_site % p.nx, y = p.probe_site / p.nx;
-    read_state<Q, ST>(p, x, y, odd != 0, f);
-    moments<Q, T>(f, rho, ux, uy);
     const unsigned k = p.counters[CNT_PROBE];
+    read_state<Q, ST>(p, x, y, odd != 0, f);
+    if constexpr (Q == 9 && sizeof(T) == 8) {  // a third of the chain
+        Eq64 m;
+        moments_f64(f, m);
+        ux = m.ux;
+        uy = m.uy;
+    } else {
+        moments<Q, T>(f, rho, ux, uy);
+    }
     p.probe_buf[2 * (k % (unsigned)p.probe_cap)] = (double)ux;
     p.probe_buf[2 * (k % (unsigned)p.probe_cap) + 1] = (double)uy;
     p.counters[CNT_PROBE] = k + 1;
