@@ -401,14 +401,19 @@ cudaError_t capture_periods(lbm_ctx* ctx, int periods, cudaGraph_t* graph, cudaG
 }
 
 // The steps of this context that line_steps takes: a D1Q3 line of a collision
-// local to the site, in FP64 or FP32 (ELBM: FP32), no probe (sampled every
-// step) and no per-kernel timing.
+// local to the site, in FP64 or FP32, no probe (sampled every step) and no
+// per-kernel timing.  ELBM in FP64 (elbm_lanes_line) up to eight sites an SM,
+// two warps each: beyond, the halo's FP64 work would cost what the launch does.
 bool line_form(const lbm_ctx* ctx, int& threads, int& halo) {
     const int coll = ctx->cfg.collision, prec = ctx->cfg.precision;
     if (ctx->Q != 3 || ctx->profiling || ctx->p.probe_buf) return false;
     if (prec != LBM_FP64 && prec != LBM_FP32) return false;
-    if (coll != LBM_LBGK && coll != LBM_MRT && coll != LBM_SMOOTH && coll != LBM_DOUBLE_MONOTONIC &&
-        !(coll == LBM_ELBM && prec == LBM_FP32))
+    if (coll == LBM_ELBM && prec == LBM_FP64) {
+        threads = 32;
+        halo = kLaneHalo;
+        return ctx->cfg.nx <= 8 * ctx->nsm;
+    }
+    if (coll != LBM_LBGK && coll != LBM_MRT && coll != LBM_SMOOTH && coll != LBM_DOUBLE_MONOTONIC && coll != LBM_ELBM)
         return false;
     return line_window(ctx->cfg.nx, ctx->nsm, threads, halo);
 }

@@ -66,6 +66,18 @@ def test_elbm_fp32(nx):
     assert all(s["elbm_solved"] + s["elbm_skipped"] + s["elbm_fallbacks"] == n for s in (sa, sb))
 
 
+@pytest.mark.parametrize("nx", [1, 2, 3, 4, 5, 31, 800, 1216, 1217])
+@pytest.mark.parametrize("bc", ["ends", "periodic"])
+def test_elbm_fp64(nx, bc):
+    """Windows of eight sites, four lanes each.  A warp's series are as long as
+    its largest deviation needs, so a site's last bits depend on its window:
+    1e-15 of alpha a step, 20 steps, both runs."""
+    cfg = dict(lattice="D1Q3", nx=nx, ny=1, bc=bc, collision="elbm", precision="fp64", beta=0.9)
+    (a, sa), (b, sb) = runs(cfg, state(cfg, 0.05), 21)
+    assert float((a - b).norm() / b.norm()) < 2 * 20 * 4 * 2.0 ** -52
+    assert all(s["elbm_solved"] + s["elbm_skipped"] + s["elbm_fallbacks"] == nx * 21 for s in (sa, sb))
+
+
 @pytest.mark.parametrize("width", [1e-7, 1e-5, 2e-3, 0.02, 0.05, 0.1, 0.2])
 def test_fp64_series(width):
     """One FP64 ELBM step at deviations in every range of the solve's series
