@@ -285,12 +285,8 @@ __global__ void __launch_bounds__(256) enstrophy_kernel(int nx, int ny, int px, 
     }
 }
 
-lbm_status reset_counters(lbm_ctx* ctx, cudaStream_t s) {
-    LBM_CK(ctx, cudaMemsetAsync(ctx->p.counters, 0, CNT_WORDS * 4 + ST_WORDS * 8, s));
-    if (ctx->p.stat_slots)
-        LBM_CK(ctx, cudaMemsetAsync(ctx->p.stat_slots, 0, kStatSlots * kStatStride * sizeof(unsigned long long), s));
-    return LBM_OK;
-}
+// 32-bit words of counters and statistics, zeroed with every new state
+constexpr int kResetWords = CNT_WORDS + 2 * ST_WORDS;
 
 }  // namespace
 
@@ -602,10 +598,9 @@ lbm_status lbm_init_device(lbm_ctx* ctx, const double* rho, const double* ux, co
     if (!ctx) return LBM_ERR_ARG;
     if (!rho || !ux || (ctx->Q == 9 && !uy)) return fail(ctx, LBM_ERR_ARG, "rho, ux (and uy for D2Q9) are required");
     const int eqkind = ctx->cfg.collision == LBM_ELBM ? LBM_EQ_ENTROPIC : ctx->cfg.equilibrium;
-    lbm_status st = reset_counters(ctx, S(stream));
-    if (st) return st;
     LBM_CK(ctx, dispatch(ctx->cfg.precision, [&](auto L) {
-               return decltype(L)::init(ctx->Q, ctx->p, rho, ux, ctx->Q == 9 ? uy : nullptr, eqkind, S(stream));
+               return decltype(L)::init(ctx->Q, ctx->p, rho, ux, ctx->Q == 9 ? uy : nullptr, eqkind, kResetWords,
+                                        S(stream));
            }));
     ctx->parity = 0;
     ctx->t = 0;
@@ -629,10 +624,8 @@ lbm_status lbm_init(lbm_ctx* ctx, const double* rho, const double* ux, const dou
 lbm_status lbm_set_state(lbm_ctx* ctx, const void* f, int dtype, void* stream) {
     if (!ctx) return LBM_ERR_ARG;
     if (!f || (dtype != LBM_DTYPE_F64 && dtype != LBM_DTYPE_F32)) return fail(ctx, LBM_ERR_ARG, "bad state buffer or dtype");
-    lbm_status st = reset_counters(ctx, S(stream));
-    if (st) return st;
     LBM_CK(ctx, dispatch(ctx->cfg.precision, [&](auto L) {
-               return decltype(L)::set_state(ctx->Q, ctx->p, f, dtype, S(stream));
+               return decltype(L)::set_state(ctx->Q, ctx->p, f, dtype, kResetWords, S(stream));
            }));
     ctx->parity = 0;
     ctx->t = 0;

@@ -522,9 +522,8 @@ lbm_status lbm_batch_set_state(lbm_batch* b, int instance, const void* f, int dt
     if (b->parity != 0) return bfail(b, LBM_ERR_STATE, "set_state needs an even step count");
     const Params& p = b->hp[instance];
     const int Q = b->L.inst[instance].Q;
-    BCK(b, cudaMemsetAsync(p.counters, 0, 256, (cudaStream_t)stream));
     BCK(b, with_format(b->precision, [&](auto LL, auto) {
-            return decltype(LL)::set_state(Q, p, f, dtype, (cudaStream_t)stream);
+            return decltype(LL)::set_state(Q, p, f, dtype, 256 / 4, (cudaStream_t)stream);
         }));
     return LBM_OK;
 }

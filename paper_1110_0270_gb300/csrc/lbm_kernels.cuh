@@ -2521,11 +2521,23 @@ __global__ void __launch_bounds__(256) cand_eval_kernel(Params p, unsigned n) {
 // ---------------------------------------------------------------------------
 // State transfer, macroscopic fields and entropy.
 // ---------------------------------------------------------------------------
+// A new state's counters (and ELBM's copies of them) start from zero: by the
+// first CTA of the kernel that sets the state, `words` 32-bit words from
+// p.counters (0: none), instead of two memsets before it.
+__device__ __forceinline__ void reset_counters_here(const Params& p, int words) {
+    if (blockIdx.x != 0 || blockIdx.y != 0) return;
+    const int t = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;
+    for (int k = t; k < words; k += nt) p.counters[k] = 0u;
+    if (words && p.stat_slots)
+        for (int k = t; k < kStatSlots * kStatStride; k += nt) p.stat_slots[k] = 0ull;
+}
+
 template <int Q, class ST>
 __global__ void init_kernel(Params p, const double* rho, const double* ux, const double* uy,
-                            int eqkind) {
+                            int eqkind, int words) {
     using T = typename ST::T;
     using L = Lat<Q>;
+    reset_counters_here(p, words);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= p.nx || y >= p.ny) return;
@@ -2558,9 +2570,10 @@ __global__ void init_uniform_kernel(Params p, double rho, double ux, double uy, 
 }
 
 template <int Q, class ST, class In>
-__global__ void set_state_kernel(Params p, const In* src) {
+__global__ void set_state_kernel(Params p, const In* src, int words) {
     using T = typename ST::T;
     using L = Lat<Q>;
+    reset_counters_here(p, words);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= p.nx || y >= p.ny) return;
@@ -2719,10 +2732,10 @@ struct Launch {
     static cudaError_t prepass(int Q, int coll, bool odd, const Params& p, cudaStream_t s);
     static cudaError_t probe(int Q, bool odd, const Params& p, cudaStream_t s);
     static cudaError_t init(int Q, const Params& p, const double* r, const double* ux,
-                            const double* uy, int eqkind, cudaStream_t s);
+                            const double* uy, int eqkind, int reset_words, cudaStream_t s);
     static cudaError_t init_uniform(int Q, const Params& p, double r, double ux, double uy,
                                     int eqkind, cudaStream_t s);
-    static cudaError_t set_state(int Q, const Params& p, const void* src, int dtype, cudaStream_t s);
+    static cudaError_t set_state(int Q, const Params& p, const void* src, int dtype, int reset_words, cudaStream_t s);
     static cudaError_t get_state(int Q, const Params& p, void* dst, int dtype, bool odd,
                                  cudaStream_t s);
     static cudaError_t macros(int Q, const Params& p, void* rho, void* u, int dtype, bool odd,
@@ -3005,12 +3018,12 @@ cudaError_t Launch<ST>::fixup(int Q, int coll, bool odd, const Params& p, cudaSt
 
 template <class ST>
 cudaError_t Launch<ST>::init(int Q, const Params& p, const double* r, const double* ux,
-                             const double* uy, int eqkind, cudaStream_t s) {
+                             const double* uy, int eqkind, int reset_words, cudaStream_t s) {
     dim3 b = site_block(Q), g = site_grid(p, b);
     if (Q == 3)
-        init_kernel<3, ST><<<g, b, 0, s>>>(p, r, ux, uy, eqkind);
+        init_kernel<3, ST><<<g, b, 0, s>>>(p, r, ux, uy, eqkind, reset_words);
     else
-        init_kernel<9, ST><<<g, b, 0, s>>>(p, r, ux, uy, eqkind);
+        init_kernel<9, ST><<<g, b, 0, s>>>(p, r, ux, uy, eqkind, reset_words);
     return cudaGetLastError();
 }
 
@@ -3026,19 +3039,19 @@ cudaError_t Launch<ST>::init_uniform(int Q, const Params& p, double r, double ux
 }
 
 template <class ST>
-cudaError_t Launch<ST>::set_state(int Q, const Params& p, const void* src, int dtype,
+cudaError_t Launch<ST>::set_state(int Q, const Params& p, const void* src, int dtype, int reset_words,
                                   cudaStream_t s) {
     dim3 b = site_block(Q), g = site_grid(p, b);
     if (dtype == LBM_DTYPE_F64) {
         if (Q == 3)
-            set_state_kernel<3, ST, double><<<g, b, 0, s>>>(p, (const double*)src);
+            set_state_kernel<3, ST, double><<<g, b, 0, s>>>(p, (const double*)src, reset_words);
         else
-            set_state_kernel<9, ST, double><<<g, b, 0, s>>>(p, (const double*)src);
+            set_state_kernel<9, ST, double><<<g, b, 0, s>>>(p, (const double*)src, reset_words);
     } else {
         if (Q == 3)
-            set_state_kernel<3, ST, float><<<g, b, 0, s>>>(p, (const float*)src);
+            set_state_kernel<3, ST, float><<<g, b, 0, s>>>(p, (const float*)src, reset_words);
         else
-            set_state_kernel<9, ST, float><<<g, b, 0, s>>>(p, (const float*)src);
+            set_state_kernel<9, ST, float><<<g, b, 0, s>>>(p, (const float*)src, reset_words);
     }
     return cudaGetLastError();
 }
