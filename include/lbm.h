@@ -316,7 +316,9 @@ typedef struct {
                          tile is tile_x x (256 / tile_x) sites, one per thread
                          (D1Q3 tiles are 256 sites of the line) */
     int ctas_per_sm;  /* CTAs per SM of each kernel, 0 = as many as fit */
-    int chunk;        /* work items claimed per queue access (1 ... 1024) */
+    int chunk;        /* work items claimed per queue access (1 ... 1024), at
+                         most: fewer where a step has less than two such
+                         claims per CTA */
     int order;        /* LBM_BATCH_ORDER_* within a step */
     int graph_steps;  /* steps per launch in the replayed graph (1 ... 4096) */
     double wait_ms;   /* limit of one wait for an instance's previous step */

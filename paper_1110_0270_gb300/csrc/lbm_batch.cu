@@ -324,8 +324,12 @@ BatchArgs make_args(const lbm_batch* b, int q, int steps) {
 cudaError_t launch_queue(lbm_batch* b, int q, int steps, cudaStream_t s) {
     if (b->L.nitems[q] == 0 || steps <= 0) return cudaSuccess;
     const int set = queue_set(q);
-    const BatchArgs a = make_args(b, q, steps);
+    BatchArgs a = make_args(b, q, steps);
     const int grid = b->grid[set];
+    // claims of `chunk` items while a step has two of them for every CTA, else
+    // fewer, so that the last round of a small batch's step is not mostly idle
+    // (32 instances, 20 steps: 4.15 -> 3.45 ms; 512 have 30 items a CTA)
+    a.chunk = std::min(a.chunk, std::max(1, a.nitems / (2 * grid)));
     return with_format(b->precision, [&](auto, auto BL) { return decltype(BL)::persistent(set, a, grid, s); });
 }
 
