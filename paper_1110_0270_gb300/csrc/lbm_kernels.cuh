@@ -2827,6 +2827,12 @@ void step_shape(const Params& p, dim3& b, dim3& g) {
     }
 }
 
+// D2Q9 ELBM in FP64 above this many sites takes CTAs of 256 sites: on large
+// lattices CTAs of 64 ran the long solve slower (every site solving: 4097^2 112 ms
+// against 91, 2049^2 33.6 against 27.1), on small ones they spread the work
+// better (400^2, 40 steps: 19.7 ms against 22.2; 257^2, 60 steps: 16.7 against 19.5).
+constexpr int64_t kElbmFlatMost = 1 << 20;
+
 template <int Q, class ST, int COLL>
 cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
     // two sites per thread where every row starts on a pair boundary (the
@@ -2850,6 +2856,11 @@ cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
                             dim3((p.nx + kLaneSites - 1) / kLaneSites), dim3(32), s, p);
     dim3 b, g;
     step_shape<Q, ST>(p, b, g);
+    if constexpr (kFlat<Q, ST> && COLL == LBM_ELBM)
+        if (!p.diffusive && (int64_t)p.nx * p.ny > kElbmFlatMost) {
+            b = dim3(256);
+            g = dim3((unsigned)(((int64_t)p.nx * p.ny + 255) / 256));
+        }
     if constexpr (Q == 9) {
         if (p.diffusive) {
             const int n = wall_sites(p);
