@@ -43,3 +43,21 @@ def test_edges(bc, sizes, prec, coll):
         # ELBM: its root to 1e-15 (FP64), or 2^-24 of alpha (FP32), a step
         tol = TOL[prec] + (0 if coll == "lbgk" else 5 * (1e-14 if prec == "fp64" else 2.0 ** -22))
         assert np.linalg.norm(g - f) < tol * np.linalg.norm(f), (nx, ny)
+
+
+def test_large_fp64_elbm():
+    """Above 2^20 sites ELBM in FP64 takes larger CTAs: a resting lattice with
+    noise in the last rows (the ragged last CTA) and beside the side walls, two
+    steps (TOL of five steps and the root's 1e-14 each)."""
+    nx, ny = 1027, 1025
+    cfg = dict(lattice="D2Q9", nx=nx, ny=ny, bc="cavity", lid_u=0.05, collision="elbm", precision="fp64", beta=0.9)
+    one = np.ones((ny, nx))
+    f0 = O.init_equilibrium(cfg, one, 0 * one, 0 * one)
+    f0[:, -3:] *= WL.lognormal_factors(f0[:, -3:].shape, 4, 1e-2)
+    f0[:, ::64, :2] *= WL.lognormal_factors(f0[:, ::64, :2].shape, 5, 1e-2)
+    lat = lbm.Lattice(cfg)
+    lat.set_state(torch.tensor(f0, device="cuda"))
+    lat.step(2)
+    f = O.step(cfg, f0, 2)
+    g = lat.get_state(torch.float64).cpu().numpy()
+    assert np.linalg.norm(g - f) < (TOL["fp64"] + 2e-14) * np.linalg.norm(f)
