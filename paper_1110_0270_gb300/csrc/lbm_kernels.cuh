@@ -2609,7 +2609,7 @@ __global__ void get_state_kernel(Params p, Out* dst, int odd) {
 }
 
 // The wall sites of one step in a kernel of their own (after the 16-bit pair
-// kernel; step_kernel carries them itself).
+// kernel and for boxes too tall for step_kernel to carry them itself).
 template <class ST, bool ODD>
 __global__ void __launch_bounds__(256) diffusive_wall_kernel(Params p) {
     pdl_enter();
@@ -2864,10 +2864,22 @@ cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
     if constexpr (Q == 9) {
         if (p.diffusive) {
             const int n = wall_sites(p);
-            if (kFlat<Q, ST>)
+            if constexpr (kFlat<Q, ST>) {
                 g.x += (n + kFlatThreads - 1) / kFlatThreads;
-            else
-                g.y += (n + (int)g.x * kBlockX * kBlockY - 1) / ((int)g.x * kBlockX * kBlockY);
+            } else {
+                const unsigned rows = (n + (int)g.x * kBlockX * kBlockY - 1) / ((int)g.x * kBlockX * kBlockY);
+                if (g.y + rows > 65535u) {
+                    // a tall box whose sites alone nearly fill the grid's y
+                    // extent: the wall sites in a kernel of their own
+                    const cudaError_t e =
+                        launch_p(odd ? step_kernel<Q, ST, COLL, true> : step_kernel<Q, ST, COLL, false>, g, b, s, p);
+                    return e != cudaSuccess
+                               ? e
+                               : launch_p(odd ? diffusive_wall_kernel<ST, true> : diffusive_wall_kernel<ST, false>,
+                                          dim3((n + 255) / 256), dim3(256), s, p);
+                }
+                g.y += rows;
+            }
             return launch_p(odd ? step_kernel<Q, ST, COLL, true, true> : step_kernel<Q, ST, COLL, false, true>, g, b, s,
                             p);
         }

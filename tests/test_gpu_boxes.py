@@ -1,0 +1,42 @@
+"""Diffusive boxes (Section 8's wall sites) at the launch shapes where the wall
+sites change kernels, against the oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle as O  # noqa: E402
+from paper_1110_0270_gb300 import lbm  # noqa: E402
+from paper_1110_0270_gb300 import workloads as WL  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def rel_error(cfg, seed, width, steps):
+    """||f - oracle|| / ||oracle|| after `steps` steps from a random flow with
+    log-normal noise of the given width."""
+    ny, nx = cfg["ny"], cfg["nx"]
+    fl = WL.random_fields(ny, nx, seed, 0.02, 0.05)
+    f0 = O.init_equilibrium(dict(cfg, collision="lbgk"), fl["rho"], fl["ux"], fl["uy"])
+    f0 = f0 * WL.lognormal_factors(f0.shape, seed + 1, width)
+    dt = torch.float64 if cfg["precision"] == "fp64" else torch.float32
+    f0 = torch.tensor(f0, dtype=dt, device="cuda")
+    lat = lbm.Lattice(cfg)
+    lat.set_state(f0)
+    lat.step(steps)
+    f = O.step(cfg, f0.double().cpu().numpy(), steps)
+    g = lat.get_state(torch.float64).cpu().numpy()
+    return float(np.linalg.norm(g - f) / np.linalg.norm(f))
+
+
+# the largest height the configuration accepts, and heights on either side of
+# the one from which the sites' own CTA rows leave no room for the wall sites'
+# (65535 rows of CTAs in all: ny / 2 for the sites and 2 (nx + ny - 2) / 256 for
+# the wall sites fill them at ny = 129052)
+@pytest.mark.parametrize("ny", [129052, 129053, 131069, 131070])
+@pytest.mark.parametrize("collision", ["lbgk", "ehrenfest"])
+def test_tall_box_fp32(ny, collision):
+    cfg = dict(lattice="D2Q9", nx=4, ny=ny, bc="diffusive", lid_u=0.1, collision=collision, precision="fp32",
+               beta=0.9, equilibrium="entropic", topk=8, delta=1e-4)
+    # three steps of about 20 operations, each 2^-24
+    assert rel_error(cfg, 3, 1e-2, 3) < 3 * 20 * 2.0 ** -24
