@@ -1586,10 +1586,11 @@ __device__ __forceinline__ void block_scan2(double& c, double& v) {
 // delta).  With S the step's sum of Delta S over the lattice (partial sums
 // of the step kernel) and R = delta0 (1 - (2 beta - 1)^2) S, the threshold
 // Delta S_0 of Eq. (EntThresh) solves L(t) = sum max(Delta S - t, 0) = R.
-// Only sites above delta matter when L(delta) > R (otherwise, and with R = 0,
-// Delta S_t = delta); then the sites whose L(Delta S) < R (the "upper" set, n
-// of them with sum S_u) give Delta S_0 = (S_u - R) / n, the root on the linear
-// piece of L below them.  Up to 32 candidates (the usual case) one warp takes
+// Only sites above delta matter when L(delta) > R (otherwise Delta S_t =
+// delta); then the sites whose L(Delta S) < R (the "upper" set, n of them with
+// sum S_u) give Delta S_0 = (S_u - R) / n, the root on the linear piece of L
+// below them.  With no upper site (R = 0: no budget, nothing to limit; or R
+// below the sums' rounding) the root is the largest value itself.  Up to 32 candidates (the usual case) one warp takes
 // them, a lane each; more go through an MSB radix descent over the FP64 bits
 // of the candidate values with per-bin counts and sums, a thread per bin.
 // (One thread walking the 256 bins of each digit, three FP64 operations of 64
@@ -1640,7 +1641,9 @@ __device__ void threshold_select_apply(const Params& p, unsigned M) {
                     nu += __shfl_xor_sync(0xffffffffu, nu, o);
                     sum += __shfl_xor_sync(0xffffffffu, sum, o);
                 }
-                if (tid == 0) s_dst = nu > 0.0 ? (sum - R) / nu : p.delta;
+                if (nu == 0.0)
+                    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+                if (tid == 0) s_dst = nu > 0.0 ? (sum - R) / nu : v;
             }
             __syncthreads();
         } else {
@@ -1667,8 +1670,8 @@ __device__ void threshold_select_apply(const Params& p, unsigned M) {
                 }
                 __syncthreads();
                 // bins from the top (thread t: bin 255 - t): the first whose lower
-                // bound b has L(b) >= R holds the boundary; the bins above it are
-                // upper
+                // bound b has L(b) >= R, with a value at or above it, holds the
+                // boundary; the bins above it are upper
                 const int d = 255 - tid;
                 const double cA = s_cntA, sA = s_sumA, c0 = (double)cnt[d], h0 = hsum[d];
                 double ci = c0, si = h0;
@@ -1676,7 +1679,7 @@ __device__ void threshold_select_apply(const Params& p, unsigned M) {
                 ci += cA;
                 si += sA;
                 const double b = __longlong_as_double((long long)(pre | ((unsigned long long)d << shift)));
-                if (si - b * ci >= R) atomicMin(&s_chosen, tid);
+                if (ci > 0.0 && si - b * ci >= R) atomicMin(&s_chosen, tid);
                 __syncthreads();
                 const int ch = s_chosen;
                 if (ch == 256 ? tid == 255 : tid == ch) {  // none: every bin is upper
@@ -1688,7 +1691,8 @@ __device__ void threshold_select_apply(const Params& p, unsigned M) {
                 __syncthreads();
                 if (ch == 256) break;
             }
-            if (tid == 0) s_dst = s_cntA > 0.0 ? (s_sumA - R) / s_cntA : p.delta;
+            if (tid == 0)
+                s_dst = s_cntA > 0.0 ? (s_sumA - R) / s_cntA : __longlong_as_double((long long)s_prefix);
             __syncthreads();
         }
         const double t0 = s_dst;
