@@ -91,16 +91,20 @@ __device__ __forceinline__ bool wait_generation(const unsigned* gen, unsigned ta
     return true;
 }
 
-// The item's sites: `rows` tiles, one site per thread in each.
+// The item's sites: `rows` tiles, one site per thread in each.  (Counting
+// ELBM's sites in every row, not the last alone, takes 1.3% of a batch's time:
+// 32 instances, 20 steps 4.09 ms against 4.04; the same with the counts in
+// shared memory or summed by warp.)
 template <int Q, class ST, int COLL>
 __device__ __forceinline__ void batch_tile(const Params& sp, const BatchItem& it, int log2x, int rows, bool odd,
-                                           int& e_code, int& e_iters) {
+                                           ElbmCount& count) {
     const int tid = threadIdx.x;
     const int th = kBatchThreads >> log2x;  // D2Q9 tile height
     typename ST::T acc = 0;                 // no reduction in the batched collisions
     for (int r = 0; r < rows; ++r) {
         const int x = Q == 9 ? it.x0 + (tid & ((1 << log2x) - 1)) : it.x0 + r * kBatchThreads + tid;
         const int y = Q == 9 ? it.y0 + r * th + (tid >> log2x) : 0;
+        int e_code = -1, e_iters = 0;
         if constexpr (kElbmWarp<ST, COLL>) {
             const bool valid = x < sp.nx && y < sp.ny;
             if (odd)
@@ -113,6 +117,7 @@ __device__ __forceinline__ void batch_tile(const Params& sp, const BatchItem& it
             else
                 site_update<Q, ST, COLL, false>(sp, x, y, e_code, e_iters, acc);
         }
+        if (COLL == LBM_ELBM) count.add(e_code, e_iters);
     }
 }
 
@@ -159,9 +164,9 @@ template <int Q, class ST, int COLL>
 __device__ __forceinline__ void batch_item(const Params& sp, const BatchItem& it, int log2x, int rows, bool odd,
                                            bool fix_only) {
     if (!fix_only) {
-        int e_code = -1, e_iters = 0;
-        batch_tile<Q, ST, COLL>(sp, it, log2x, rows, odd, e_code, e_iters);
-        if (COLL == LBM_ELBM) elbm_stats(sp, e_code, e_iters);
+        ElbmCount count;
+        batch_tile<Q, ST, COLL>(sp, it, log2x, rows, odd, count);
+        if (COLL == LBM_ELBM) elbm_stats(sp, count);
     } else {
         batch_fixup<Q, ST, COLL>(sp, odd);
     }

@@ -893,13 +893,25 @@ __device__ __forceinline__ void elbm_update(const Params& p, int x, int y, bool 
     }
 }
 
+// The ELBM counts of one thread's sites, up to 64 (the batched kernels' rows):
+// how many were solved, skipped and without a root (a byte each, by ElbmOut's
+// code; -1: no site), their iterations and the largest iteration count.
+struct ElbmCount {
+    unsigned n = 0u, iters = 0u, itmax = 0u;
+    __device__ __forceinline__ void add(int code, int it) {
+        if (code >= 0) n += 1u << (8 * code);
+        iters += (unsigned)it;
+        itmax = max(itmax, (unsigned)it);
+    }
+};
+
 // Warp-aggregated ELBM counters (all 32 lanes of the warp call this).
-__device__ __forceinline__ void elbm_stats(const Params& p, int e_code, int e_iters) {
-    unsigned solved = __reduce_add_sync(0xffffffffu, e_code == 0 ? 1u : 0u);
-    unsigned skipped = __reduce_add_sync(0xffffffffu, e_code == 1 ? 1u : 0u);
-    unsigned fallback = __reduce_add_sync(0xffffffffu, e_code == 2 ? 1u : 0u);
-    unsigned iters = __reduce_add_sync(0xffffffffu, (unsigned)e_iters);
-    unsigned itmax = __reduce_max_sync(0xffffffffu, (unsigned)e_iters);
+__device__ __forceinline__ void elbm_stats(const Params& p, const ElbmCount& c) {
+    unsigned solved = __reduce_add_sync(0xffffffffu, c.n & 255u);
+    unsigned skipped = __reduce_add_sync(0xffffffffu, (c.n >> 8) & 255u);
+    unsigned fallback = __reduce_add_sync(0xffffffffu, c.n >> 16);
+    unsigned iters = __reduce_add_sync(0xffffffffu, c.iters);
+    unsigned itmax = __reduce_max_sync(0xffffffffu, c.itmax);
     if (lane_id() == 0) {
         unsigned long long* st =
             p.stat_slots ? p.stat_slots + ((blockIdx.y * gridDim.x + blockIdx.x) % kStatSlots) * kStatStride : p.stats;
@@ -911,6 +923,11 @@ __device__ __forceinline__ void elbm_stats(const Params& p, int e_code, int e_it
         if (itmax && itmax > *(volatile unsigned long long*)&st[ST_ELBM_ITERS_MAX])
             atomicMax(&st[ST_ELBM_ITERS_MAX], (unsigned long long)itmax);
     }
+}
+__device__ __forceinline__ void elbm_stats(const Params& p, int e_code, int e_iters) {
+    ElbmCount c;
+    c.add(e_code, e_iters);
+    elbm_stats(p, c);
 }
 
 // CTA-wide sums of a and b added to partial-sum slot (linear block id mod
