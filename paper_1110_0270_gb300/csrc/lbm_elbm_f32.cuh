@@ -326,8 +326,9 @@ __device__ __forceinline__ Ff ff_g(Ff x, float& ln) {
     int e = 0;
     Ff num = x;
     if (!near) {
-        // 2^-e w in [0.7, 1.42], less 1
-        e = (int)((__float_as_uint(w.h) + 0x4afb0du) >> 23) - 127;  // m < 1.4142 keeps the exponent
+        // 2^-e w in [0.7, 1.42], less 1: the exponent counts up where the fraction
+        // passes that of sqrt(2) (0x3504f3; 0x4afb0d = 2^23 - 0x3504f3)
+        e = (int)((__float_as_uint(w.h) + 0x4afb0du) >> 23) - 127;
         const float sc = __uint_as_float((unsigned)(127 - e) << 23);
         num = two_sum(fmul(w.h, sc), -1.f);
         num = fast_two_sum(num.h, fmaf(w.l, sc, num.l));
@@ -455,7 +456,12 @@ __device__ __noinline__ ElbmSite<Q> elbm_f32_far(const Params& p, ElbmSite<Q> in
             exists = true;
             const float next = a - step;
             const bool close = dH > 0.f && fabsf(step) <= 1e-4f * a && next < hi0.h;
-            settled = fine && close;
+            // what a last step leaves is H'' / (2 H') step^2.  A root next to
+            // a = hi0 has one small 1 + x = w there, H'' / H' <= 1 / (a w |ln w|),
+            // and w > 1.2e-4 (w (1 - ln w) > 1e-3 by the margin above): below
+            // 450 step^2 / a, 0.44 x 2^-24 a for steps up to 2^-17 a (measured up
+            // to there: 0.28 x 2^-24 of alpha)
+            settled = fine && close && fabsf(step) <= 0x1p-17f * a;
             if (!settled) a = close || (dH > 0.f && next > lo && next < hi) ? next : 0.5f * (lo + hi);
             if (close && !fine) {  // FP32 rounding may have put a bound on the wrong side
                 fine = true;
