@@ -230,13 +230,14 @@ def run_variants(n_side, steps, warmup, fma_per_s=None):
             if fma_per_s and (coll == "elbm" or precision == "fp64"):
                 out[f"{coll}/{precision}"]["fp64_fma_slots_per_site"] = round(fma_per_s / (mlups * 1e6), 1)
             if coll == "elbm":
-                # the root finder's work: FP64 parabola steps per solved site
-                # (after the FP32 pre-iterations) and the share of each outcome
+                # the root finder's work: iterations per solved site (FP64
+                # storage: parabola steps after the FP32 pre-iterations; FP32 and
+                # 16-bit storage: one) and the share of each outcome
                 st = lat.stats()
                 tot = max(1, st["elbm_solved"] + st["elbm_skipped"] + st["elbm_fallbacks"])
                 out[f"{coll}/{precision}"]["elbm"] = {
-                    "fp64_steps_per_solved": round(st["elbm_iters_total"] / max(1, st["elbm_solved"]), 4),
-                    "fp64_steps_max": st["elbm_iters_max"], "solved_frac": round(st["elbm_solved"] / tot, 4),
+                    "iters_per_solved": round(st["elbm_iters_total"] / max(1, st["elbm_solved"]), 4),
+                    "iters_max": st["elbm_iters_max"], "solved_frac": round(st["elbm_solved"] / tot, 4),
                     "skipped_frac": round(st["elbm_skipped"] / tot, 4),
                     "fallback_frac": round(st["elbm_fallbacks"] / tot, 6)}
             del lat
@@ -257,8 +258,9 @@ def run_elbm_loaded(n_side, steps=5):
     """ELBM with every site solved: the 4097^2 cavity started from the random
     velocity field of random_start (the variants table starts from rest,
     where the near-equilibrium skip takes most sites), FP32 and FP64 storage:
-    MLUPS, FP64 parabola steps per solved site (after the FP32
-    pre-iterations) and the share of solved / skipped / fallback sites."""
+    MLUPS, iterations per solved site (FP64 parabola steps after the FP32
+    pre-iterations; one for a site solved in FP32) and the share of solved /
+    skipped / fallback sites."""
     import torch
     from paper_1110_0270_gb300 import lbm
     out = {}
@@ -275,7 +277,7 @@ def run_elbm_loaded(n_side, steps=5):
         tot = max(1, d["elbm_solved"] + d["elbm_skipped"] + d["elbm_fallbacks"])
         out[precision] = {"mlups": round(n_side * n_side * steps / (ms * 1e-3) / 1e6, 1),
                           "ms_per_step": round(ms / steps, 3),
-                          "fp64_steps_per_solved": round(d["elbm_iters_total"] / max(1, d["elbm_solved"]), 4),
+                          "iters_per_solved": round(d["elbm_iters_total"] / max(1, d["elbm_solved"]), 4),
                           "solved_frac": round(d["elbm_solved"] / tot, 4),
                           "skipped_frac": round(d["elbm_skipped"] / tot, 4),
                           "fallback_frac": round(d["elbm_fallbacks"] / tot, 6)}

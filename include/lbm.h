@@ -139,6 +139,12 @@ typedef struct {
     int topk;        /* Ehrenfest: at most this many sites per step (>= 0) */
     double delta;    /* Ehrenfest / median threshold on Delta S (>= 0) */
     double s_e, s_eps, s_q; /* MRT relaxation rates of C1 */
+    /* ELBM's FP64 solve, which FP64 storage runs at every site.  FP32 and
+     * 16-bit storage solve in FP32 (f* - f as sums of two floats, within
+     * 2^-40 f*; alpha to its FP32 rounding, 2^-24, or better) and take these
+     * three only at the few sites outside that form's range: velocities above
+     * 0.4, densities outside 2^-20 ... 2^20, f below 2^-12 f* or above 5 f*,
+     * or a root too close to the edge of its existence or to the skip. */
     double elbm_eps;        /* ELBM stopping tolerance (> 0), e.g. 1e-15 */
     int elbm_max_iter;      /* ELBM parabola iterations (>= 1), e.g. 20 */
     int elbm_norm;          /* LBM_NORM_* in the stopping rule */
@@ -158,9 +164,11 @@ typedef struct {
                                   LBM_DOUBLE_MONOTONIC, LBM_ENSEMBLE, which act
                                   on every site) */
     uint64_t elbm_solved;      /* ELBM sites that ran the root finder */
-    uint64_t elbm_skipped;     /* ELBM sites with Delta S < 1e-15 */
+    uint64_t elbm_skipped;     /* ELBM sites with Delta S < 1e-15 (FP32 and
+                                  16-bit storage: 1e-15 + 2^-48 rho) */
     uint64_t elbm_fallbacks;   /* ELBM sites without a non-trivial root */
-    uint64_t elbm_iters_total; /* parabola iterations, summed */
+    uint64_t elbm_iters_total; /* FP64 parabola iterations, summed; a site
+                                  solved in FP32 counts one */
     uint64_t elbm_iters_max;   /* largest iteration count at one site */
     uint64_t diverged;         /* 1 once a non-finite or non-positive rho is seen */
     uint64_t overflow;         /* 1 if a candidate list overflowed (never with
@@ -297,7 +305,7 @@ lbm_status lbm_last_candidates(lbm_ctx* ctx, double* ds, int32_t* site, int32_t*
  * instance's limiter fix-up (Ehrenfest selection, median filter) before
  * publishing it.  Three kernels, on parallel stream branches: the streaming
  * collisions (LBGK, positivity, MRT), the limiters (Ehrenfest, median) and
- * ELBM (its FP64 root finder needs far more registers).
+ * ELBM (its root finder needs far more registers).
  * graph_steps steps of both are captured once, at creation, into a CUDA
  * graph that lbm_batch_step replays.  Every wait is bounded (wait_ms): one
  * that runs out stops the launch and the next status check returns
