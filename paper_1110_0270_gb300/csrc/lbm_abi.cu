@@ -74,7 +74,7 @@ void fill_params(const lbm_config* cfg, int nsm, Params& p) {
     p.ny = cfg->ny;
     p.periodic_x = cfg->bc == LBM_BC_PERIODIC || cfg->bc == LBM_BC_CHANNEL;
     p.periodic_y = cfg->bc == LBM_BC_PERIODIC;
-    p.eq = cfg->equilibrium;
+    p.eq = cfg->collision == LBM_ELBM ? LBM_EQ_ENTROPIC : cfg->equilibrium;
     p.lid_u = (cfg->bc == LBM_BC_CAVITY || cfg->bc == LBM_BC_CHANNEL) ? cfg->lid_u : 0.0;
     p.diffusive = cfg->bc == LBM_BC_DIFFUSIVE;
     p.wall_u = p.diffusive ? cfg->lid_u : 0.0;
@@ -597,7 +597,7 @@ lbm_status lbm_init_device(lbm_ctx* ctx, const double* rho, const double* ux, co
                            void* stream) {
     if (!ctx) return LBM_ERR_ARG;
     if (!rho || !ux || (ctx->Q == 9 && !uy)) return fail(ctx, LBM_ERR_ARG, "rho, ux (and uy for D2Q9) are required");
-    const int eqkind = ctx->cfg.collision == LBM_ELBM ? LBM_EQ_ENTROPIC : ctx->cfg.equilibrium;
+    const int eqkind = ctx->p.eq;
     LBM_CK(ctx, dispatch(ctx->cfg.precision, [&](auto L) {
                return decltype(L)::init(ctx->Q, ctx->p, rho, ux, ctx->Q == 9 ? uy : nullptr, eqkind, kResetWords,
                                         S(stream));
@@ -690,7 +690,7 @@ lbm_status lbm_macros(lbm_ctx* ctx, void* rho, void* u, int dtype, void* stream)
 lbm_status lbm_entropy(lbm_ctx* ctx, double* H_total_host, double* dS_dev, void* stream) {
     if (!ctx) return LBM_ERR_ARG;
     if (!H_total_host && !dS_dev) return fail(ctx, LBM_ERR_ARG, "no output requested");
-    const int eqkind = ctx->cfg.collision == LBM_ELBM ? LBM_EQ_ENTROPIC : ctx->cfg.equilibrium;
+    const int eqkind = ctx->p.eq;
     double* H = ctx->p.scratch_d;
     LBM_CK(ctx, cudaMemsetAsync(H, 0, sizeof(double), S(stream)));
     LBM_CK(ctx, dispatch(ctx->cfg.precision, [&](auto L) {

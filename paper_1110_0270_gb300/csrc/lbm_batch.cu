@@ -406,9 +406,6 @@ lbm_status create_batch(const lbm_config* cfgs, int n, const lbm_batch_opts& o, 
         p.plane = I.plane;
         p.plane32 = (int)I.plane;
         p.pitch = I.pitch;
-        // ELBM always uses the entropic equilibrium; storing it here makes the
-        // uniform initialisation pick the right one
-        if (c->collision == LBM_ELBM) p.eq = LBM_EQ_ENTROPIC;
         p.median_inv = 0.0;  // the batched median filter reads the step's Delta S field
         p.counters = (unsigned*)(b->base + I.cnt_off);
         p.stats = (unsigned long long*)(b->base + I.cnt_off + CNT_WORDS * 4);

@@ -40,3 +40,15 @@ def test_tall_box_fp32(ny, collision):
                beta=0.9, equilibrium="entropic", topk=8, delta=1e-4)
     # three steps of about 20 operations, each 2^-24
     assert rel_error(cfg, 3, 1e-2, 3) < 3 * 20 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("equilibrium", ["poly", "entropic", "poly_std"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_elbm_walls_are_entropic(precision, equilibrium):
+    """ELBM's equilibria are entropic whatever the configuration names, at the
+    wall sites too (a fast top wall, where the kinds differ most)."""
+    cfg = dict(lattice="D2Q9", nx=37, ny=29, bc="diffusive", lid_u=0.3, collision="elbm", precision=precision,
+               beta=0.9, equilibrium=equilibrium)
+    # five steps of 40 (20) operations and the root's 1e-14 (2^-22)
+    tol = 5 * (40 * 2.0 ** -53 + 1e-14) if precision == "fp64" else 5 * (20 * 2.0 ** -24 + 2.0 ** -22)
+    assert rel_error(cfg, 3, 1e-2, 5) < tol
