@@ -1047,9 +1047,9 @@ __device__ __forceinline__ void step_body(const Params& p, typename ST::T* save)
     if constexpr (kFlat<Q, ST>) {
         const unsigned s = blockIdx.x * blockDim.x + threadIdx.x;
         if constexpr (WALLS) {
-            const unsigned b = (unsigned)(p.nx * p.ny + kFlatThreads - 1) / kFlatThreads;
+            const unsigned b = (unsigned)(p.nx * p.ny + blockDim.x - 1) / blockDim.x;
             if (blockIdx.x >= b) {
-                wall_site<ST, ODD>(p, (int)(s - b * kFlatThreads));
+                wall_site<ST, ODD>(p, (int)(s - b * blockDim.x));
                 return;
             }
         }
@@ -2849,10 +2849,11 @@ void step_shape(const Params& p, dim3& b, dim3& g) {
 }
 
 // D2Q9 ELBM in FP64 above this many sites takes CTAs of 256 sites: on large
-// lattices CTAs of 64 ran the long solve slower (every site solving: 4097^2 112 ms
-// against 91, 2049^2 33.6 against 27.1), on small ones they spread the work
-// better (400^2, 40 steps: 19.7 ms against 22.2; 257^2, 60 steps: 16.7 against 19.5).
-constexpr int64_t kElbmFlatMost = 1 << 20;
+// lattices CTAs of 64 run the long solve slower, on small ones they spread the
+// work better.  Every site solving, us a step with 64 against 256: 257^2 411,
+// 457; 400^2 967, 1047; 513^2 1501, 1582; 600^2 2022, 2020; 700^2 2830, 2688;
+// 850^2 4279, 3884; 1025^2 6393, 5602; 2049^2 26680, 21989.
+constexpr int64_t kElbmFlatMost = 600 * 600;
 
 template <int Q, class ST, int COLL>
 cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
@@ -2878,7 +2879,7 @@ cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
     dim3 b, g;
     step_shape<Q, ST>(p, b, g);
     if constexpr (kFlat<Q, ST> && COLL == LBM_ELBM)
-        if (!p.diffusive && (int64_t)p.nx * p.ny > kElbmFlatMost) {
+        if ((int64_t)p.nx * p.ny > kElbmFlatMost) {
             b = dim3(256);
             g = dim3((unsigned)(((int64_t)p.nx * p.ny + 255) / 256));
         }
@@ -2886,7 +2887,7 @@ cudaError_t launch_step_q(bool odd, const Params& p, cudaStream_t s) {
         if (p.diffusive) {
             const int n = wall_sites(p);
             if constexpr (kFlat<Q, ST>) {
-                g.x += (n + kFlatThreads - 1) / kFlatThreads;
+                g.x += (n + b.x - 1) / b.x;
             } else {
                 const unsigned rows = (n + (int)g.x * kBlockX * kBlockY - 1) / ((int)g.x * kBlockX * kBlockY);
                 if (g.y + rows > 65535u) {

@@ -52,3 +52,23 @@ def test_elbm_walls_are_entropic(precision, equilibrium):
     # five steps of 40 (20) operations and the root's 1e-14 (2^-22)
     tol = 5 * (40 * 2.0 ** -53 + 1e-14) if precision == "fp64" else 5 * (20 * 2.0 ** -24 + 2.0 ** -22)
     assert rel_error(cfg, 3, 1e-2, 5) < tol
+
+
+# FP64 ELBM takes CTAs of 64 sites up to 360000 and of 256 above, the wall sites
+# behind the others in CTAs of the same size
+@pytest.mark.parametrize("nx,ny", [(600, 600), (601, 600), (1030, 1025)])
+@pytest.mark.parametrize("bc", ["cavity", "diffusive"])
+def test_fp64_elbm_cta_sizes(nx, ny, bc):
+    cfg = dict(lattice="D2Q9", nx=nx, ny=ny, bc=bc, lid_u=0.05, collision="elbm", precision="fp64", beta=0.9)
+    one = np.ones((ny, nx))
+    f0 = O.init_equilibrium(cfg, one, 0 * one, 0 * one)
+    # noise where the last CTA and the walls are
+    f0[:, -4:] *= WL.lognormal_factors(f0[:, -4:].shape, 4, 1e-2)
+    f0[:, ::64, :3] *= WL.lognormal_factors(f0[:, ::64, :3].shape, 5, 1e-2)
+    lat = lbm.Lattice(cfg)
+    lat.set_state(torch.tensor(f0, device="cuda"))
+    lat.step(3)
+    g = lat.get_state(torch.float64).cpu().numpy()
+    f = O.step(cfg, f0, 3)
+    # three steps of 40 operations, each 2^-53, and the root's 1e-14
+    assert np.linalg.norm(g - f) < (3 * 40 * 2.0 ** -53 + 3e-14) * np.linalg.norm(f)
