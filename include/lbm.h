@@ -239,7 +239,11 @@ lbm_status lbm_get_state(lbm_ctx* ctx, void* f, int dtype, void* stream);
 /* Advances nsteps >= 0 steps.  Allocates nothing.  Pairs of steps that start
  * at an even step count replay the context's graph (one launch instead of
  * two to four, which matters for small lattices); the rest, and every step
- * while kernel tracing is on, are launched one by one. */
+ * while kernel tracing is on, are launched one by one.  D1Q3 lines of up to
+ * 240 sites an SM (FP64 ELBM: 8), in FP64 or FP32, of a collision that needs
+ * nothing but the site, without a probe, advance up to 12 (2) steps per launch
+ * instead, through the context's scratch; such a call may also be captured
+ * into a caller's graph. */
 lbm_status lbm_step(lbm_ctx* ctx, int nsteps, void* stream);
 
 /* Density rho[ny][nx] and velocity u[2][ny][nx] (u_x plane then u_y plane;
