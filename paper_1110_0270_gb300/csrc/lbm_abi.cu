@@ -319,8 +319,9 @@ lbm_status initial_mean(lbm_ctx* ctx, cudaStream_t s) {
 namespace {
 
 // The kernels of one step with counter slot `cslot` and A-A parity `odd`;
-// save: where the step keeps its pre-collision state (step_save), after_kernel
-// as for read_out.
+// save: where the step keeps its pre-collision state (step_save); after_kernel
+// as for read_out (false: the step's first kernel starts after the stream's
+// last operation has ended).
 cudaError_t enqueue_one_step(lbm_ctx* ctx, bool odd, int cslot, cudaStream_t s, void* save = nullptr,
                              bool after_kernel = true) {
     const int coll = ctx->cfg.collision;
@@ -336,9 +337,9 @@ cudaError_t enqueue_one_step(lbm_ctx* ctx, bool odd, int cslot, cudaStream_t s, 
     if (e == cudaSuccess)
         e = traced(ctx, LBM_KERNEL_STEP, s, [&] {
             return dispatch(ctx->cfg.precision, [&](auto L) {  // diffusive wall sites included
-                if (!save) return decltype(L)::step(ctx->Q, coll, odd, q, s);
                 Params r = q;
                 if (!after_kernel) r.pdl = 0;
+                if (!save) return decltype(L)::step(ctx->Q, coll, odd, r, s);
                 return decltype(L)::step_save(ctx->Q, coll, odd, r, save, s);
             });
         });
@@ -431,15 +432,20 @@ bool capturing(cudaStream_t s) {
 }
 
 // n (even, >= 2) steps from an even step count: pairs of launches through the
-// staging area (3 nx doubles, otherwise scratch of lbm_init and lbm_enstrophy) and back.
-cudaError_t enqueue_line(lbm_ctx* ctx, int n, int threads, int halo, cudaStream_t s) {
-    const Params& p = ctx->p;
+// staging area (3 nx doubles, otherwise scratch of lbm_init and lbm_enstrophy)
+// and back.  apart: the first launch starts after the stream's last kernel has
+// ended.
+cudaError_t enqueue_line(lbm_ctx* ctx, int n, int threads, int halo, bool apart, cudaStream_t s) {
+    Params p = ctx->p;
     for (int k = 0; k < n;) {
         const int m = std::min(n - k, 2 * halo), a = m / 2, b = m - a;
+        p.pdl = k == 0 && apart ? 0 : 1;
         cudaError_t e = dispatch(ctx->cfg.precision, [&](auto L) {
+            Params q = p;
+            q.pdl = 1;
             cudaError_t r = decltype(L)::line(ctx->cfg.collision, p, p.f, p.plane, ctx->staging, p.nx, threads, a, halo, s);
             return r != cudaSuccess ? r
-                                    : decltype(L)::line(ctx->cfg.collision, p, ctx->staging, p.nx, p.f, p.plane, threads,
+                                    : decltype(L)::line(ctx->cfg.collision, q, ctx->staging, p.nx, p.f, p.plane, threads,
                                                         b, halo, s);
         });
         if (e != cudaSuccess) return e;
@@ -665,6 +671,15 @@ lbm_status lbm_step(lbm_ctx* ctx, int nsteps, void* stream) {
     if (line && rest < kLineLeast32 && ctx->cfg.precision == LBM_FP32 && ctx->cfg.collision != LBM_ELBM)
         line = capturing(S(stream));
     if (line) {
+        // between a single step and the line form in FP64 no launch ahead: the
+        // CTAs of one, placed while the other's run, fill the SMs that the
+        // smaller grid leaves free with several each, and the kernels after them
+        // keep that uneven placement, which CTAs of enough FP64 work to fill an
+        // SM's pipe take double the time for (smooth limiter, calls of three steps,
+        // us a step: 36,000 sites 24.9, 16.5 this way, 17.3 by single steps;
+        // 14,000 12.3, 9.7; CTAs of one or two warps are faster launched ahead,
+        // 3,000 sites 8.5 against 9.0)
+        const bool apart = ctx->cfg.precision == LBM_FP64 && threads > 64;
         if (ctx->parity == 1) {
             LBM_CK(ctx, enqueue_one_step(ctx, true, 1, S(stream)));
             ctx->parity = 0;
@@ -672,9 +687,15 @@ lbm_status lbm_step(lbm_ctx* ctx, int nsteps, void* stream) {
             k = 1;
         }
         const int n = (nsteps - k) & ~1;
-        LBM_CK(ctx, enqueue_line(ctx, n, threads, halo, S(stream)));
+        LBM_CK(ctx, enqueue_line(ctx, n, threads, halo, apart && k == 1, S(stream)));
         ctx->t += n;
         k += n;
+        if (k < nsteps) {
+            LBM_CK(ctx, enqueue_one_step(ctx, false, 0, S(stream), nullptr, !apart));
+            ctx->parity = 1;
+            ctx->t += 1;
+            ++k;
+        }
     }
     const bool use_graph = ctx->graph_exec && !ctx->profiling;
     while (k < nsteps) {

@@ -3011,11 +3011,16 @@ cudaError_t launch_line(const Params& p, const void* src, int64_t sp, void* dst,
                         int halo, cudaStream_t s) {
     if constexpr (COLL == LBM_ELBM && sizeof(typename ST::T) == 8) {
         constexpr int own = kLaneSites - 2 * kLaneHalo;
-        return launch_pdl(elbm_lanes_line<ST>, (p.nx + own - 1) / own, 32, s, p, src, sp, dst, dp, steps);
+        const int g = (p.nx + own - 1) / own;
+        if (p.pdl) return launch_pdl(elbm_lanes_line<ST>, g, 32, s, p, src, sp, dst, dp, steps);
+        elbm_lanes_line<ST><<<g, 32, 0, s>>>(p, src, sp, dst, dp, steps);
+        return cudaGetLastError();
     }
     if constexpr (kLineForm<ST, COLL>) {
-        const int own = threads - 2 * halo;
-        return launch_pdl(line_steps<ST, COLL>, (p.nx + own - 1) / own, threads, s, p, src, sp, dst, dp, steps, halo);
+        const int own = threads - 2 * halo, g = (p.nx + own - 1) / own;
+        if (p.pdl) return launch_pdl(line_steps<ST, COLL>, g, threads, s, p, src, sp, dst, dp, steps, halo);
+        line_steps<ST, COLL><<<g, threads, 0, s>>>(p, src, sp, dst, dp, steps, halo);
+        return cudaGetLastError();
     }
     return cudaErrorInvalidValue;
 }
