@@ -2040,6 +2040,18 @@ __device__ __forceinline__ void eval_then_select(const Params& p) {
         if (M > (unsigned)p.cand_cap) M = (unsigned)p.cand_cap;
         if (small && M > (blockDim.x >> 4) && M <= 2 * blockDim.x && settle_all_taken<Q, ST, ODD, COLL>(p, M)) return;
     }
+    if (COLL == LBM_THRESHOLD && M == 0) {
+        // nothing above delta, so no threshold to look for: only the step's sums
+        // are cleared (an 800-site line in FP32 10.3 us a step, 4.6 this way)
+        if (blockIdx.x != 0) return;
+        for (int k = threadIdx.x; k < kRedSlots; k += blockDim.x) p.red[k] = 0.0;
+        if (threadIdx.x == 0) {
+            p.counters[CNT_NVALID] = 0u;
+            p.counters[CNT_NSEL] = 0u;
+            *p.lim_E = p.delta;  // as threshold_select_apply leaves it
+        }
+        return;
+    }
     if (M <= (blockDim.x >> 4)) {
         // few screened sites (the usual case): the first CTA evaluates them
         // all, one 16-lane group each, and selects without the ticket and
