@@ -2033,6 +2033,11 @@ __device__ __forceinline__ void eval_then_select(const Params& p) {
     // every CTA costs the usual short list 1 us (257^2 cavity with a few screened
     // sites 11.8 us a step against 10.3, in 16-bit storage 13.1 against 11.8)
     constexpr bool kAhead = sizeof(typename ST::S) == 8;
+    // CTAs beyond one per SM (launch_fixup_q) take part only in a list of more
+    // than one round, and of more than settle_all_taken tries
+    const unsigned base = (unsigned)p.pipe_ctas / 8;
+    const unsigned round = max(2 * blockDim.x, base * (blockDim.x >> 4));
+    if (blockIdx.x >= base && p.counters[p.cslot] <= round) return;
     if (kAhead && small) {
         if (settle_all_taken<Q, ST, ODD, COLL>(p, M)) return;
     } else {
@@ -2149,12 +2154,13 @@ __device__ __forceinline__ void eval_then_select(const Params& p) {
         }
         return;
     }
+    const unsigned ncta = M <= round && gridDim.x > base ? base : gridDim.x;
     unsigned n = 0;
     // one record per 16-lane group
-    const unsigned groups = gridDim.x * (blockDim.x >> 4);
+    const unsigned groups = ncta * (blockDim.x >> 4);
     const unsigned g0 = blockIdx.x * (blockDim.x >> 4) + (threadIdx.x >> 4);
-    for (unsigned base = 0; base < M; base += groups) {
-        const unsigned j = base + g0;
+    for (unsigned j0 = 0; j0 < M; j0 += groups) {
+        const unsigned j = j0 + g0;
         const double d = delta_s_group<Q, ST>(p, j, j < M);
         if (j < M && (threadIdx.x & 15) == 0) {
             const bool c = d > p.delta;
@@ -2166,7 +2172,7 @@ __device__ __forceinline__ void eval_then_select(const Params& p) {
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(&p.counters[CNT_NVALID], n);
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&p.counters[CNT_DONE], 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) s_last = atomicAdd(&p.counters[CNT_DONE], 1u) == ncta - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
@@ -2961,13 +2967,38 @@ cudaError_t launch_step_c(int coll, bool odd, const Params& p, cudaStream_t s) {
     return cudaErrorInvalidValue;
 }
 
+constexpr int64_t kTwoSites = 1 << 17, kApartSites = 1 << 19;
+
 template <int Q, class ST>
 cudaError_t launch_fixup_q(int coll, bool odd, const Params& p, cudaStream_t s, int nsm) {
     // the candidate count is only known on the device: a fixed grid of one
     // CTA per SM strides over the list
-    if (coll == LBM_EHRENFEST)
-        return launch_p(odd ? ehrenfest_eval_select<Q, ST, true> : ehrenfest_eval_select<Q, ST, false>, nsm,
-                        256, s, p);
+    if (coll == LBM_EHRENFEST || coll == LBM_MRT_LIMITER) {
+        Params q = p;
+        unsigned g = nsm;
+        // Launched ahead, the CTAs go to whatever SMs the step's last wave leaves
+        // first, several to one, and a long list takes up to twice the time.  A
+        // second CTA per SM, which short lists do not use, evens that out where
+        // it costs the step nothing: FP32 boxes with the wall sites in the step,
+        // and 2^17 to 2^19 sites; above, the kernel follows the step, which is
+        // long against a launch (16-bit boxes have the wall kernel between).
+        // Every site above delta, us a step: FP32 box 513^2 1518 -> 1070, cavity
+        // 513^2 1513 -> 1053, 1025^2 15724 -> 9890, 16-bit cavity 513^2 1460 ->
+        // 1041; a few, FP32 cavity: 513^2 12.3 both ways, 1025^2 36 -> 32.  (FP64
+        // box of 129^2 with two CTAs per SM 10.5 -> 12.4, FP32 cavity of 257^2
+        // not launched ahead 11.2 -> 11.9.)
+        const bool walls = Q == 9 && p.diffusive;
+        const int64_t N = (int64_t)p.nx * p.ny;
+        if ((walls && sizeof(typename ST::S) == 4) || (N > kTwoSites && N <= kApartSites))
+            g = 2 * nsm;
+        else if (N > kApartSites && !(walls && sizeof(typename ST::S) == 2))
+            q.pdl = 0;
+        void (*k)(Params) =
+            coll == LBM_EHRENFEST
+                ? (odd ? ehrenfest_eval_select<Q, ST, true> : ehrenfest_eval_select<Q, ST, false>)
+                : (odd ? mrt_limiter_eval_select<Q, ST, true> : mrt_limiter_eval_select<Q, ST, false>);
+        return launch_p(k, g, 256, s, q);
+    }
     // the field-free median filter takes one candidate per CTA and round:
     // four CTAs per SM, so that thousands of candidates overlap their FP64
     // window evaluations (with few, the CTAs without one exit at once)
@@ -2978,9 +3009,6 @@ cudaError_t launch_fixup_q(int coll, bool odd, const Params& p, cudaStream_t s, 
         return launch_p(odd ? median_fixup<Q, ST, true> : median_fixup<Q, ST, false>, nsm, 256, s, p);
     if (coll == LBM_THRESHOLD)
         return launch_p(odd ? threshold_eval_select<Q, ST, true> : threshold_eval_select<Q, ST, false>, nsm,
-                        256, s, p);
-    if (coll == LBM_MRT_LIMITER)
-        return launch_p(odd ? mrt_limiter_eval_select<Q, ST, true> : mrt_limiter_eval_select<Q, ST, false>, nsm,
                         256, s, p);
     if (coll == LBM_ENSEMBLE_LAGGED) return launch_p(ensemble_finalize<ST>, 1, 256, s, p);
     return cudaSuccess;
