@@ -85,15 +85,13 @@ void fill_params(const lbm_config* cfg, int nsm, Params& p) {
     p.lid_u_f = (float)p.lid_u;
     p.delta_f = (float)cfg->delta;
     const double snu = 2.0 * p.beta;
-    p.mrt.e = cfg->s_e / 36.0;
-    p.mrt.eps = cfg->s_eps / 36.0;
-    p.mrt.q = cfg->s_q / 12.0;
-    p.mrt.nu = snu / 4.0;
-    p.mrt_f = {(float)p.mrt.e, (float)p.mrt.eps, (float)p.mrt.q, (float)p.mrt.nu};
     {
+        // C1_k / N_k
+        const double re = cfg->s_e / 36.0, reps = cfg->s_eps / 36.0, rq = cfg->s_q / 12.0, rnu = snu / 4.0;
+        p.mrt_f = {(float)re, (float)reps, (float)rq, (float)rnu};
         // e = 3 (A + 2 D), eps = -3 (2 A + D); axis rows -e - 2 eps, diagonal rows 2 e + eps
-        const double e = 3.0 * p.mrt.e, ep = -3.0 * p.mrt.eps;
-        p.mrt64 = {-e - 4.0 * ep, -2.0 * (e + ep), 2.0 * (e + ep), 4.0 * e + ep, 3.0 * p.mrt.q, 6.0 * p.mrt.q, p.mrt.nu};
+        const double e = 3.0 * re, ep = -3.0 * reps;
+        p.mrt64 = {-e - 4.0 * ep, -2.0 * (e + ep), 2.0 * (e + ep), 4.0 * e + ep, 3.0 * rq, 6.0 * rq, rnu};
         p.two_beta = snu;
         p.mrt2_c = (snu - 1.0) / 4.0;
     }

@@ -361,18 +361,6 @@ __device__ __forceinline__ float pow_lim(float x, float k) {
 __device__ __forceinline__ double rel_dev(double d, double q) { return d / q; }
 __device__ __forceinline__ float rel_dev(float d, float q) { return __fdividef(d, q); }
 
-template <int Q, class T>
-__device__ __forceinline__ T delta_s_t(const T* f, const T* feq) {
-    T s = T(0);
-    bool neg = false;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        neg |= (f[i] < T(0)) || !(feq[i] > T(0));
-        s += feq[i] * gfun<T>(rel_dev(f[i] - feq[i], feq[i]));
-    }
-    return neg ? T(INFINITY) : s;
-}
-
 // Limiter screens (FP32, no FP64 instruction: GB300's FP64 rate is a small
 // fraction of its FP32 rate).  Each returns true when the site may exceed
 // delta and needs the exact FP64 Delta S.  With d = f - f*, x = d / f* and
@@ -508,26 +496,25 @@ __device__ __forceinline__ void conserve_mass(T rho, T* F) {
 // A_2 = I + (s_nu - 1)/4 (r4 r4^T + r5 r5^T), r4 = v_x^2 - v_y^2,
 // r5 = v_x v_y per velocity, so F = f - A_2 (f - f*) =
 // f* + (1 - s_nu)/4 (m4 r4 + m5 r5), m = r . (f - f*).
-template <class T>
-__device__ __forceinline__ void mrt2_d2q9(const T* f, const T* feq, T om, T* F) {
+__device__ __forceinline__ void mrt2_d2q9(const float* f, const float* feq, float om, float* F) {
     using L = Lat<9>;
-    T m4 = T(0), m5 = T(0);
+    float m4 = 0.f, m5 = 0.f;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        const T d = f[i] - feq[i];
+        const float d = f[i] - feq[i];
         const int r4 = L::cx(i) * L::cx(i) - L::cy(i) * L::cy(i), r5 = L::cx(i) * L::cy(i);
         if (r4 > 0) m4 += d;
         if (r4 < 0) m4 -= d;
         if (r5 > 0) m5 += d;
         if (r5 < 0) m5 -= d;
     }
-    const T c = (T(1) - om) * T(0.25);
+    const float c = (1.f - om) * 0.25f;
     m4 *= c;
     m5 *= c;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int r4 = L::cx(i) * L::cx(i) - L::cy(i) * L::cy(i), r5 = L::cx(i) * L::cy(i);
-        F[i] = feq[i] + T(r4) * m4 + T(r5) * m5;
+        F[i] = feq[i] + float(r4) * m4 + float(r5) * m5;
     }
 }
 
@@ -565,26 +552,19 @@ __device__ __forceinline__ bool positivity(const T* feq, T* F) {
 // 6, 12, 4, 4) the inverse is M1^T N^-1, so
 // F = f - M1^T (C1 N^-1) M1 (f - f*).  The conserved rows contribute zero
 // (f and f* share rho and rho u) and are skipped.  rate[k] = C1_k / N_k.
-template <class T>
-__device__ __forceinline__ void mrt_d2q9(const T* f, const T* feq, const MrtRates& rd,
-                                         const MrtRatesF& rf, T* F) {
-    // rates in T (FP32 copies avoid per-site FP64 conversions)
-    struct {
-        T e, eps, q, nu;
-    } r = {sizeof(T) == 8 ? T(rd.e) : T(rf.e), sizeof(T) == 8 ? T(rd.eps) : T(rf.eps),
-           sizeof(T) == 8 ? T(rd.q) : T(rf.q), sizeof(T) == 8 ? T(rd.nu) : T(rf.nu)};
-    T d[9];
+__device__ __forceinline__ void mrt_d2q9(const float* f, const float* feq, const MrtRatesF& r, float* F) {
+    float d[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) d[i] = f[i] - feq[i];
     // rows of M1 in the paper numbering (rest, E, SE, S, SW, W, NW, N, NE)
-    T se = d[2] + d[4] + d[6] + d[8];  // diagonals
-    T ax = d[1] + d[3] + d[5] + d[7];  // axis
-    T e = T(-4) * d[0] - ax + T(2) * se;
-    T ep = T(4) * d[0] - T(2) * ax + se;
-    T qx = T(-2) * d[1] + d[2] - d[4] + T(2) * d[5] - d[6] + d[8];
-    T qy = -d[2] + T(2) * d[3] - d[4] + d[6] - T(2) * d[7] + d[8];
-    T pxx = d[1] - d[3] + d[5] - d[7];
-    T pxy = -d[2] + d[4] - d[6] + d[8];
+    float se = d[2] + d[4] + d[6] + d[8];  // diagonals
+    float ax = d[1] + d[3] + d[5] + d[7];  // axis
+    float e = -4.f * d[0] - ax + 2.f * se;
+    float ep = 4.f * d[0] - 2.f * ax + se;
+    float qx = -2.f * d[1] + d[2] - d[4] + 2.f * d[5] - d[6] + d[8];
+    float qy = -d[2] + 2.f * d[3] - d[4] + d[6] - 2.f * d[7] + d[8];
+    float pxx = d[1] - d[3] + d[5] - d[7];
+    float pxy = -d[2] + d[4] - d[6] + d[8];
     e *= r.e;
     ep *= r.eps;
     qx *= r.q;
@@ -592,15 +572,15 @@ __device__ __forceinline__ void mrt_d2q9(const T* f, const T* feq, const MrtRate
     pxx *= r.nu;
     pxy *= r.nu;
     // F_i = f_i - sum_k M1[k][i] * m_k
-    F[0] = f[0] - (T(-4) * e + T(4) * ep);
-    F[1] = f[1] - (-e - T(2) * ep - T(2) * qx + pxx);
-    F[2] = f[2] - (T(2) * e + ep + qx - qy - pxy);
-    F[3] = f[3] - (-e - T(2) * ep + T(2) * qy - pxx);
-    F[4] = f[4] - (T(2) * e + ep - qx - qy + pxy);
-    F[5] = f[5] - (-e - T(2) * ep + T(2) * qx + pxx);
-    F[6] = f[6] - (T(2) * e + ep - qx + qy - pxy);
-    F[7] = f[7] - (-e - T(2) * ep - T(2) * qy - pxx);
-    F[8] = f[8] - (T(2) * e + ep + qx + qy + pxy);
+    F[0] = f[0] - (-4.f * e + 4.f * ep);
+    F[1] = f[1] - (-e - 2.f * ep - 2.f * qx + pxx);
+    F[2] = f[2] - (2.f * e + ep + qx - qy - pxy);
+    F[3] = f[3] - (-e - 2.f * ep + 2.f * qy - pxx);
+    F[4] = f[4] - (2.f * e + ep - qx - qy + pxy);
+    F[5] = f[5] - (-e - 2.f * ep + 2.f * qx + pxx);
+    F[6] = f[6] - (2.f * e + ep - qx + qy - pxy);
+    F[7] = f[7] - (-e - 2.f * ep - 2.f * qy - pxx);
+    F[8] = f[8] - (2.f * e + ep + qx + qy + pxy);
 }
 
 // ELBM (Section 3).  S_f(alpha) = S(f + alpha Delta) - S(f), Delta = f* - f,

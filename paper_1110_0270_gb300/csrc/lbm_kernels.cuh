@@ -298,10 +298,11 @@ __device__ __forceinline__ void collide_site(const Params& p, int x, int y, cons
         equilibrium<Q, T>(p.eq, rho, ux, uy, feq);
         if (COLL == LBM_EHRENFEST || COLL == LBM_MEDIAN || COLL == LBM_MRT_LIMITER)
             limiter_screen<Q, T, COLL == LBM_MRT_LIMITER ? LBM_EHRENFEST : COLL>(p, x, y, f, feq, rho);
-        if (COLL == LBM_MRT && Q == 9) {
-            mrt_d2q9<T>(f, feq, p.mrt, p.mrt_f, F);
-        } else if (COLL == LBM_MRT2 && Q == 9) {
-            mrt2_d2q9<T>(f, feq, sizeof(T) == 8 ? T(2.0 * p.beta) : T(2) * T(p.beta_f), F);
+        // (D2Q9 in FP64: mrt_f64, mrt2_f64)
+        if constexpr (COLL == LBM_MRT && Q == 9 && sizeof(T) == 4) {
+            mrt_d2q9(f, feq, p.mrt_f, F);
+        } else if constexpr (COLL == LBM_MRT2 && Q == 9 && sizeof(T) == 4) {
+            mrt2_d2q9(f, feq, 2.f * p.beta_f, F);
         } else {
             lbgk<Q, T>(f, feq, sizeof(T) == 8 ? T(p.beta) : T(p.beta_f), F);
         }
@@ -1777,7 +1778,7 @@ __device__ __forceinline__ void rewrite_selected(const Params& p, int site, cons
         if constexpr (COLL == LBM_MRT_LIMITER && Q == 9) {
             // Section 5's MRT limiter: the selected site takes A_2, not f*
             T F[Q];
-            mrt2_d2q9<T>(f, feq, sizeof(T) == 8 ? T(2.0 * p.beta) : T(2) * T(p.beta_f), F);
+            mrt2_d2q9(f, feq, 2.f * p.beta_f, F);
             conserve_mass<Q, T>(rho, F);
             rewrite_site<Q, ST, ODD>(p, site, F);
         } else {
@@ -2378,20 +2379,6 @@ __global__ void __launch_bounds__(256) median_fixup(Params p) {
     median_apply<Q, ST, ODD>(p, blockIdx.x * (blockDim.x >> 4) + (threadIdx.x >> 4), gridDim.x * (blockDim.x >> 4));
 }
 
-// Median filter, second kernel, without a Delta S field (|1 - 2 beta| >= 1/16
-// for FP32 and FP64 storage, >= 1/4 for 16-bit): the step ran LBGK and the Ehrenfest
-// screen at every site, so a window site's pre-collision state is either
-// its record (a screened site) or is recovered from its post-collision one
-// (delta_s_lanes with inv = 1 / (1 - 2 beta)); its Delta S is FP64.  One
-// candidate per CTA and round (one 16-lane group per window site, so the
-// narrow FP64 pipe of several SMs shares the work); the first lane of the
-// centre group takes the lower median and the new populations.  With at
-// most kMedDirect screened sites every window site is looked up in the
-// list, no window reads a post-collision state that a rewrite changes, and
-// each CTA rewrites its candidate at once; with more, the windows are all
-// recovered from the lattice, and the rewrites wait for every window of
-// the step: each selected site's coefficient goes to its record and the
-// last CTA to finish (ticket after a fence) writes the new populations.
 // The post-collision state of a median candidate whose pre-collision state f
 // gets the homothety with coefficient phi before the LBGK collision.
 template <int Q, class ST>
@@ -2428,6 +2415,20 @@ struct MedWin {
 };
 constexpr unsigned kMedDirect = 64;
 
+// Median filter, second kernel, without a Delta S field (|1 - 2 beta| >= 1/16
+// for FP32 and FP64 storage, >= 1/4 for 16-bit): the step ran LBGK and the Ehrenfest
+// screen at every site, so a window site's pre-collision state is either
+// its record (a screened site) or is recovered from its post-collision one
+// (delta_s_lanes with inv = 1 / (1 - 2 beta)); its Delta S is FP64.  One
+// candidate per CTA and round (one 16-lane group per window site, so the
+// narrow FP64 pipe of several SMs shares the work); the first lane of the
+// centre group takes the lower median and the new populations.  With at
+// most kMedDirect screened sites every window site is looked up in the
+// list, no window reads a post-collision state that a rewrite changes, and
+// each CTA rewrites its candidate at once; with more, the windows are all
+// recovered from the lattice, and the rewrites wait for every window of
+// the step: each selected site's coefficient goes to its record and the
+// last CTA to finish (ticket after a fence) writes the new populations.
 template <int Q, class ST, bool ODD>
 __global__ void __launch_bounds__(256) median_recon_fixup(Params p) {
     pdl_enter();

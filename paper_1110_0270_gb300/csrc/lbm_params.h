@@ -9,9 +9,6 @@ namespace lbm {
 
 // MRT rates divided by the squared row norms of M1 (Section 5):
 // e: s_e/36, eps: s_eps/36, q: s_q/12, nu: s_nu/4 with s_nu = 2 beta.
-struct MrtRates {
-    double e, eps, q, nu;
-};
 struct MrtRatesF {
     float e, eps, q, nu;
 };
@@ -62,7 +59,6 @@ struct Params {
     float beta_f, lid_u_f, delta_f;  // FP32 copies (no FP64 conversions per site)
     int topk;
     double delta;
-    MrtRates mrt;
     MrtRatesF mrt_f;
     Mrt64 mrt64;
     double two_beta, mrt2_c;         // 2 beta, (2 beta - 1) / 4 (no per-site FP64 arithmetic)
