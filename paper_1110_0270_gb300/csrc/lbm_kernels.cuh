@@ -2978,21 +2978,21 @@ cudaError_t launch_fixup_q(int coll, bool odd, const Params& p, cudaStream_t s, 
         Params q = p;
         unsigned g = nsm;
         // Launched ahead, the CTAs go to whatever SMs the step's last wave leaves
-        // first, several to one, and a long list takes up to twice the time.  A
-        // second CTA per SM, which short lists do not use, evens that out where
+        // first, several to one, and a long list takes up to half as long again.
+        // A second CTA per SM, which short lists do not use, evens that out where
         // it costs the step nothing: FP32 boxes with the wall sites in the step,
-        // and 2^17 to 2^19 sites; above, the kernel follows the step, which is
-        // long against a launch (16-bit boxes have the wall kernel between).
-        // Every site above delta, us a step: FP32 box 513^2 1518 -> 1070, cavity
-        // 513^2 1513 -> 1053, 1025^2 15724 -> 9890, 16-bit cavity 513^2 1460 ->
-        // 1041; a few, FP32 cavity: 513^2 12.3 both ways, 1025^2 36 -> 32.  (FP64
-        // box of 129^2 with two CTAs per SM 10.5 -> 12.4, FP32 cavity of 257^2
-        // not launched ahead 11.2 -> 11.9.)
+        // and 2^17 to 2^19 sites; in larger FP64 boxes the kernel follows the
+        // step, which is long against a launch.  Every site above delta, us a
+        // step: FP32 box 513^2 1518 -> 1070, cavity 513^2 1513 -> 1053, 16-bit
+        // cavity 513^2 1460 -> 1041, FP64 box 1025^2 14,157 -> 10,286; a few, FP32
+        // cavity 513^2 12.3 both ways.  (FP64 box of 129^2 with two CTAs per SM
+        // 10.5 -> 12.4; not launched ahead, the FP32 cavity of 257^2 11.2 -> 11.9,
+        // and two streams of 4097^2 cavities 2% slower from host to host.)
         const bool walls = Q == 9 && p.diffusive;
         const int64_t N = (int64_t)p.nx * p.ny;
         if ((walls && sizeof(typename ST::S) == 4) || (N > kTwoSites && N <= kApartSites))
             g = 2 * nsm;
-        else if (N > kApartSites && !(walls && sizeof(typename ST::S) == 2))
+        else if (walls && sizeof(typename ST::S) == 8 && N > kApartSites)
             q.pdl = 0;
         void (*k)(Params) =
             coll == LBM_EHRENFEST

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("nx,ny,bc", [(301, 203, "diffusive"), (401, 333, "cavity"), (401, 333, "diffusive"),
-                                      (731, 725, "cavity")])
+                                      (731, 725, "cavity"), (731, 725, "diffusive")])
 @pytest.mark.parametrize("collision,precision", [("ehrenfest", "fp32"), ("ehrenfest", "fp64"), ("mrt_limiter", "fp32")])
 @pytest.mark.parametrize("rounds,more", [(0, 40), (0, 600), (1, -1), (1, 0), (1, 1), (2, 1)])
 def test_lists(nx, ny, bc, collision, precision, rounds, more):
