@@ -18,7 +18,7 @@
 // Three kernels per storage format, each on its own stream branch: the
 // streaming collisions (LBGK, positivity, MRT: no fix-up, few registers,
 // many resident CTAs), the limiters (Ehrenfest, median: their fix-ups in
-// the kernel) and ELBM (its FP64 root finder needs far more registers).
+// the kernel) and ELBM (its root finder needs far more registers).
 // A work item is `rows` tiles of one instance (tile_x x 256 / tile_x sites,
 // one per thread, for D2Q9; 256 sites of the line for D1Q3): a CTA that
 // stays on one instance and step keeps its parameters and skips the wait.
@@ -91,10 +91,7 @@ __device__ __forceinline__ bool wait_generation(const unsigned* gen, unsigned ta
     return true;
 }
 
-// The item's sites: `rows` tiles, one site per thread in each.  (Counting
-// ELBM's sites in every row, not the last alone, takes 1.3% of a batch's time:
-// 32 instances, 20 steps 4.09 ms against 4.04; the same with the counts in
-// shared memory or summed by warp.)
+// The item's sites: `rows` tiles, one site per thread in each.
 template <int Q, class ST, int COLL>
 __device__ __forceinline__ void batch_tile(const Params& sp, const BatchItem& it, int log2x, int rows, bool odd,
                                            ElbmCount& count) {
@@ -117,7 +114,7 @@ __device__ __forceinline__ void batch_tile(const Params& sp, const BatchItem& it
             else
                 site_update<Q, ST, COLL, false>(sp, x, y, e_code, e_iters, acc);
         }
-        if (COLL == LBM_ELBM) count.add(e_code, e_iters);
+        if (COLL == LBM_ELBM) count.add(sp, e_code, e_iters);
     }
 }
 
@@ -166,7 +163,7 @@ __device__ __forceinline__ void batch_item(const Params& sp, const BatchItem& it
     if (!fix_only) {
         ElbmCount count;
         batch_tile<Q, ST, COLL>(sp, it, log2x, rows, odd, count);
-        if (COLL == LBM_ELBM) elbm_stats(sp, count);
+        if (COLL == LBM_ELBM) count.flush(sp);
     } else {
         batch_fixup<Q, ST, COLL>(sp, odd);
     }

@@ -894,47 +894,74 @@ __device__ __forceinline__ void elbm_update(const Params& p, int x, int y, bool 
     }
 }
 
-// The ELBM counts of one thread's sites, up to 64 (the batched kernels' rows):
-// how many were solved, skipped and without a root (a byte each, by ElbmOut's
-// code; -1: no site), their iterations and the largest iteration count.
-struct ElbmCount {
-    unsigned n = 0u, iters = 0u, itmax = 0u;
-    __device__ __forceinline__ void add(int code, int it) {
-        if (code >= 0) n += 1u << (8 * code);
-        iters += (unsigned)it;
-        itmax = max(itmax, (unsigned)it);
-    }
-};
+// Where this CTA's ELBM counters go.
+__device__ __forceinline__ unsigned long long* elbm_counters(const Params& p) {
+    return p.stat_slots ? p.stat_slots + ((blockIdx.y * gridDim.x + blockIdx.x) % kStatSlots) * kStatStride : p.stats;
+}
+// The largest iteration count only grows: most callers find theirs no larger.
+__device__ __forceinline__ void elbm_iters_max(unsigned long long* st, unsigned it) {
+    if (it > *(volatile unsigned long long*)&st[ST_ELBM_ITERS_MAX])
+        atomicMax(&st[ST_ELBM_ITERS_MAX], (unsigned long long)it);
+}
 
 // Warp-aggregated ELBM counters (all 32 lanes of the warp call this).
-__device__ __forceinline__ void elbm_stats(const Params& p, const ElbmCount& c) {
-    unsigned solved = __reduce_add_sync(0xffffffffu, c.n & 255u);
-    unsigned skipped = __reduce_add_sync(0xffffffffu, (c.n >> 8) & 255u);
-    unsigned fallback = __reduce_add_sync(0xffffffffu, c.n >> 16);
-    unsigned iters = __reduce_add_sync(0xffffffffu, c.iters);
-    unsigned itmax = __reduce_max_sync(0xffffffffu, c.itmax);
+__device__ __forceinline__ void elbm_stats(const Params& p, int e_code, int e_iters) {
+    unsigned solved = __reduce_add_sync(0xffffffffu, e_code == 0 ? 1u : 0u);
+    unsigned skipped = __reduce_add_sync(0xffffffffu, e_code == 1 ? 1u : 0u);
+    unsigned fallback = __reduce_add_sync(0xffffffffu, e_code == 2 ? 1u : 0u);
+    unsigned iters = __reduce_add_sync(0xffffffffu, (unsigned)e_iters);
+    unsigned itmax = __reduce_max_sync(0xffffffffu, (unsigned)e_iters);
     if (lane_id() == 0) {
-        unsigned long long* st =
-            p.stat_slots ? p.stat_slots + ((blockIdx.y * gridDim.x + blockIdx.x) % kStatSlots) * kStatStride : p.stats;
+        unsigned long long* st = elbm_counters(p);
         if (solved) atomicAdd(&st[ST_ELBM_SOLVED], (unsigned long long)solved);
         if (skipped) atomicAdd(&st[ST_ELBM_SKIPPED], (unsigned long long)skipped);
         if (fallback) atomicAdd(&st[ST_ELBM_FALLBACK], (unsigned long long)fallback);
         if (iters) atomicAdd(&st[ST_ELBM_ITERS], (unsigned long long)iters);
-        // (the largest count only grows: most warps find theirs no larger)
-        if (itmax && itmax > *(volatile unsigned long long*)&st[ST_ELBM_ITERS_MAX])
-            atomicMax(&st[ST_ELBM_ITERS_MAX], (unsigned long long)itmax);
+        if (itmax) elbm_iters_max(st, itmax);
     }
 }
-__device__ __forceinline__ void elbm_stats(const Params& p, int e_code, int e_iters) {
-    ElbmCount c;
-    c.add(e_code, e_iters);
-    elbm_stats(p, c);
-}
+
+// The same for several sites of a thread (the batched kernels' rows, up to 64),
+// in one register across them: how many were solved, skipped and without a
+// root (a byte each, by ElbmOut's code; -1: no site) and how many took one
+// iteration, the usual count; a site with more adds its own by itself.  (With
+// the iterations and the largest count in registers too, a batch of 32
+// instances took 4.09 ms for 20 steps; 4.06 this way, 4.03 counting the last
+// row alone.)
+struct ElbmCount {
+    unsigned n = 0u;
+    __device__ __forceinline__ void add(const Params& p, int code, int it) {
+        if (code >= 0) n += 1u << (8 * code);
+        if (it == 1) n += 1u << 24;
+        if (it > 1) {
+            unsigned long long* st = elbm_counters(p);
+            atomicAdd(&st[ST_ELBM_ITERS], (unsigned long long)it);
+            elbm_iters_max(st, (unsigned)it);
+        }
+    }
+    // (all 32 lanes of the warp call this)
+    __device__ __forceinline__ void flush(const Params& p) const {
+        unsigned solved = __reduce_add_sync(0xffffffffu, n & 255u);
+        unsigned skipped = __reduce_add_sync(0xffffffffu, (n >> 8) & 255u);
+        unsigned fallback = __reduce_add_sync(0xffffffffu, (n >> 16) & 255u);
+        unsigned iters = __reduce_add_sync(0xffffffffu, n >> 24);
+        if (lane_id() == 0) {
+            unsigned long long* st = elbm_counters(p);
+            if (solved) atomicAdd(&st[ST_ELBM_SOLVED], (unsigned long long)solved);
+            if (skipped) atomicAdd(&st[ST_ELBM_SKIPPED], (unsigned long long)skipped);
+            if (fallback) atomicAdd(&st[ST_ELBM_FALLBACK], (unsigned long long)fallback);
+            if (iters) {
+                atomicAdd(&st[ST_ELBM_ITERS], (unsigned long long)iters);
+                elbm_iters_max(st, 1u);
+            }
+        }
+    }
+};
 
 // CTA-wide sums of a and b added to partial-sum slot (linear block id mod
 // kRedSlots) of p.red (and, with two, of p.red + kRedSlots).  Every thread
 // of the CTA calls it.  The CTA's sum is formed in T (FP32 in the 16/32-bit
-// modes: 256 values, relative error ~5e-7 at worst, far below the FP32
+// modes: at most 256 values, relative error ~5e-7 at worst, far below the FP32
 // parity bound) by two shuffle stages, and one FP64 atomic per CTA adds it:
 // GB300's narrow FP64 pipe would otherwise hold every CTA at its end.
 template <class T>
@@ -2038,7 +2065,7 @@ __device__ __forceinline__ void eval_then_select(const Params& p) {
     // than one round, and of more than settle_all_taken tries
     const unsigned base = (unsigned)p.pipe_ctas / 8;
     const unsigned round = max(2 * blockDim.x, base * (blockDim.x >> 4));
-    if (blockIdx.x >= base && p.counters[p.cslot] <= round) return;
+    if (blockIdx.x >= base && min(p.counters[p.cslot], (unsigned)p.cand_cap) <= round) return;
     if (kAhead && small) {
         if (settle_all_taken<Q, ST, ODD, COLL>(p, M)) return;
     } else {
@@ -2860,8 +2887,10 @@ inline dim3 site_grid(const Params& p, dim3 block) {
 inline dim3 site_block(int Q) { return Q == 3 ? dim3(256, 1) : dim3(kBlockX, kBlockY); }
 
 // A line up to this long takes four lanes per site in FP64 ELBM: the groups of
-// lanes run a shorter chain on four times the warps (800 sites: 20.6 us a step
-// against 49; 20000 sites, where the warps fill the FP64 pipes: 58 us against 55).
+// lanes run a shorter chain on four times the warps, which longer lines cannot
+// spread over more SMs.  us a step by threads and by lanes, near rest / flow:
+// 8000 sites 21, 15 / 37, 19; 14000 23, 17 / 37, 28; 16000 21, 19 / 40, 40; 18000
+// 24, 20 / 40, 42; 32000 24, 26 / 61, 63; 60000 27, 37 / 126, 105.
 constexpr int kElbmLaneMost = 16000;
 
 // CTA and grid of the one-site step kernel.
