@@ -198,8 +198,8 @@ def time_steps(lat, steps, warmup, dist=None, profile=False, sampler=None):
 
 def run_variants(n_side, steps, warmup, fma_per_s=None):
     """MLUPS and fraction of HBM peak per collision x precision (one GPU).
-    The FP64-bound ones (ELBM's root solve, FP64 storage) also get their cost
-    in FP64 FMA issue slots per site at the measured FMA rate."""
+    The FP64-bound ones (FP64 storage) also get their cost in FP64 FMA issue
+    slots per site at the measured FMA rate."""
     import torch
     from paper_1110_0270_gb300 import lbm
     hbm, _ = peaks()
@@ -227,7 +227,7 @@ def run_variants(n_side, steps, warmup, fma_per_s=None):
                 "kernel_ms": round(kstep, 5), "steps": k}
             if prof["fixup"][0]:
                 out[f"{coll}/{precision}"]["fixup_ms"] = round(prof["fixup"][1] / prof["fixup"][0], 5)
-            if fma_per_s and (coll == "elbm" or precision == "fp64"):
+            if fma_per_s and precision == "fp64":
                 out[f"{coll}/{precision}"]["fp64_fma_slots_per_site"] = round(fma_per_s / (mlups * 1e6), 1)
             if coll == "elbm":
                 # the root finder's work: iterations per solved site (FP64

@@ -19,9 +19,10 @@
  * Collisions (lbm_config.collision):
  *   LBM_LBGK        F = f + 2 beta (f* - f)                  (Eq. CollisionIntegral)
  *   LBM_ELBM        F = f + alpha beta (f* - f), alpha the non-trivial root of
- *                   S(f + alpha (f* - f)) = S(f), entropic f*; parabola root
- *                   finder in FP64 (Section 3.3, Eqs. NewCondition,
- *                   Stopping, ConvergenceTwo)
+ *                   S(f + alpha (f* - f)) = S(f), entropic f* (Section 3.3,
+ *                   Eqs. NewCondition, Stopping, ConvergenceTwo): parabola root
+ *                   finder in FP64 for FP64 storage; FP32 and 16-bit storage
+ *                   as described at lbm_config.elbm_eps
  *   LBM_EHRENFEST   LBGK, except that among the sites with Delta S > delta the
  *                   k (= topk) largest jump to f* (Section 4, Ehrenfests'
  *                   regularisation); Delta S = sum f ln(f/f*) (Eq. DelS)
@@ -503,8 +504,8 @@ lbm_status lbm_ehrenfest_step_noalloc(const lbm_config* cfg, void* f, int nsteps
  * current GPU: *dfma_flops = FP64 fused multiply-add rate in FLOP/s (2 per
  * FMA), *log_per_s = FP64 log() evaluations per second, each from one timed
  * launch after a warm-up launch on `stream` (synchronised).  These are the
- * ceilings of the step kernels bound by the FP64 pipe (the ELBM root solve,
- * FP64 storage).  Either output may be NULL, not both (LBM_ERR_ARG).
+ * ceilings of the step kernels bound by the FP64 pipe (FP64 storage, ELBM's
+ * root solve in it above all).  Either output may be NULL, not both (LBM_ERR_ARG).
  * Allocates and frees 8 bytes of device memory; LBM_ERR_CUDA on failure.
  * ------------------------------------------------------------------------- */
 lbm_status lbm_fp64_rates(double* dfma_flops, double* log_per_s, void* stream);

@@ -66,7 +66,7 @@ extern "C" lbm_status lbm_ehrenfest_step_noalloc(const lbm_config* cfg, void* f,
                                                  void* stream) {
     if (!cfg || !f || nsteps < 0 || (nsteps & 1)) return LBM_ERR_ARG;
     // the checks of lbm_create, then what this entry point does not cover:
-    // other collisions and the diffusive walls (their wall kernel)
+    // other collisions and diffusive walls
     if (check_config(cfg)) return LBM_ERR_ARG;
     if (cfg->collision != LBM_EHRENFEST || cfg->bc == LBM_BC_DIFFUSIVE) return LBM_ERR_ARG;
     const int Q = cfg->lattice == LBM_D1Q3 ? 3 : 9;
