@@ -1075,9 +1075,10 @@ __device__ __forceinline__ void step_body(const Params& p, typename ST::T* save)
     if constexpr (kFlat<Q, ST>) {
         const unsigned s = blockIdx.x * blockDim.x + threadIdx.x;
         if constexpr (WALLS) {
-            const unsigned b = (unsigned)(p.nx * p.ny + blockDim.x - 1) / blockDim.x;
-            if (blockIdx.x >= b) {
-                wall_site<ST, ODD>(p, (int)(s - b * blockDim.x));
+            // (CTAs of 64 or 256 sites: no division by their size)
+            const unsigned first = ((unsigned)(p.nx * p.ny) + blockDim.x - 1) & ~(blockDim.x - 1);
+            if (s >= first) {
+                wall_site<ST, ODD>(p, (int)(s - first));
                 return;
             }
         }
